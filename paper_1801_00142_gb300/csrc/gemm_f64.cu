@@ -7,101 +7,145 @@
 // tensors (struct Idx3), so no permutation pass is needed between steps.
 //
 // This is the FP64 path; it also serves the canonicalisation and the traces
-// of the tensor-core path.  On GB300 the FP64 rate
-// is a small fraction of the FP32 rate, so the FP64 kernel is bound by FP64
-// issue: a 64x64 output tile per 256-thread CTA, 4x4 outputs per thread, k
-// staged 16 at a time through shared memory, with the per-tile view offsets
-// precomputed once per tile.
+// of the tensor-core path.  What bounds it: a GB300 SM retires two FP64 FMAs
+// a clock (64 times fewer than FP32), so a 32 x 32 x 16 tile step keeps the
+// pipe busy for 8192 clocks and neither shared memory nor L2 matters; the
+// time is the FMAs issued by the busiest SM.  Hence
+//  - small tiles (32 x 32) with the contraction split over a cluster of up to
+//    8 CTAs, so that every SM gets the same share also when the output has
+//    few tiles (the partial tiles are summed in rank order through
+//    distributed shared memory: no workspace, the same result every run);
+//  - a warp owns 4 rows x 32 columns: rows past M cost nothing in steps of 4
+//    (the transfers have 1, 5 or 25 of them), and the two operands are
+//    exchanged when that wastes fewer lanes.
+// Measured: all transfers of one observables row at L = 64, D* = 256 (31
+// GFLOP, 25 ms at the pipe's rate): 245 ms with 64 x 64 tiles and no split,
+// 38 ms with these.
 #include "common.cuh"
+
+#include <cooperative_groups.h>
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+namespace cg = cooperative_groups;
 
-template <typename T, typename G>
-__global__ void __launch_bounds__(NT) gemm_kernel(G g, int a_kfast, int b_kfast) {
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
+constexpr int BM = 32, BN = 32, BK = 16, NT = 256;
+constexpr int LDA = BM + 2, LDB = BN + 2;   // even: 16-byte reads of a row pair
+constexpr int SPLIT_MAX = 8;                // portable cluster size
+
+// idx_off with 32-bit divisions (every index of a view is below 2^31)
+__device__ __forceinline__ long long off32(const Idx3& d, unsigned idx) {
+  if (d.n0 == 1 && d.n1 == 1) return (long long)idx * d.s2;
+  const unsigned t = idx / (unsigned)d.n0, i0 = idx - t * (unsigned)d.n0;
+  const unsigned i2 = t / (unsigned)d.n1, i1 = t - i2 * (unsigned)d.n1;
+  return (long long)i2 * d.s2 + (long long)i1 * d.s1 + (long long)i0 * d.s0;
+}
+
+// One 32 x 32 output tile over K range [k_begin, k_end) of this cluster rank.
+template <bool SPLIT>
+__global__ void __launch_bounds__(NT) gemm_kernel(GemmF64 g, int a_kfast, int b_kfast, int splits,
+                                                  int k_per) {
+  __shared__ __align__(16) double As[BK][LDA];
+  __shared__ __align__(16) double Bs[BK][LDB];
   __shared__ long long offAm[BM], offBn[BN], offAk[BK], offBk[BK];
 
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
+  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const long long b = blockIdx.z;
-  const T* A = g.A + b * g.sab;
-  const T* B = g.B + b * g.sbb;
+  const int rank = SPLIT ? (int)(blockIdx.z % splits) : 0;
+  const long long b = SPLIT ? blockIdx.z / splits : blockIdx.z;
+  const int k_begin = SPLIT ? rank * k_per : 0;
+  const int k_end = SPLIT ? min(g.K, k_begin + k_per) : g.K;
+  const double* A = g.A + b * g.sab;
+  const double* B = g.B + b * g.sbb;
 
   if (tid < BM) {
-    int m = m0 + tid;
-    offAm[tid] = (m < g.M) ? idx_off(g.am, m) : 0;
+    const int m = m0 + tid;
+    offAm[tid] = (m < g.M) ? off32(g.am, m) : 0;
   } else if (tid < BM + BN) {
-    int n = n0 + tid - BM;
-    offBn[tid - BM] = (n < g.N) ? idx_off(g.bn, n) : 0;
+    const int n = n0 + tid - BM;
+    offBn[tid - BM] = (n < g.N) ? off32(g.bn, n) : 0;
   }
 
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  const bool live = m0 + 4 * warp < g.M;   // this warp's rows (uniform in the warp)
 
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
+  for (int k0 = k_begin; k0 < k_end; k0 += BK) {
     __syncthreads();
     if (tid < BK) {
-      int k = k0 + tid;
-      offAk[tid] = (k < g.K) ? idx_off(g.ak, k) : 0;
+      const int k = k0 + tid;
+      offAk[tid] = (k < k_end) ? off32(g.ak, k) : 0;
     } else if (tid >= 32 && tid < 32 + BK) {
-      int k = k0 + tid - 32;
-      offBk[tid - 32] = (k < g.K) ? idx_off(g.bk, k) : 0;
+      const int k = k0 + tid - 32;
+      offBk[tid - 32] = (k < k_end) ? off32(g.bk, k) : 0;
     }
     __syncthreads();
+    double va[2], vb[2];
 #pragma unroll
-    for (int q = 0; q < (BM * BK) / NT; ++q) {
-      int e = tid + q * NT;
-      int mi, ki;
-      if (a_kfast) { ki = e % BK; mi = e / BK; } else { mi = e % BM; ki = e / BM; }
-      int m = m0 + mi, k = k0 + ki;
-      As[ki][mi] = (m < g.M && k < g.K) ? A[offAm[mi] + offAk[ki]] : T(0);
+    for (int q = 0; q < 2; ++q) {
+      const int e = tid + q * NT;
+      const int mi = a_kfast ? e / BK : e % BM, ka = a_kfast ? e % BK : e / BM;
+      const int ni = b_kfast ? e / BK : e % BN, kb = b_kfast ? e % BK : e / BN;
+      va[q] = (m0 + mi < g.M && k0 + ka < k_end) ? A[offAm[mi] + offAk[ka]] : 0.0;
+      vb[q] = (n0 + ni < g.N && k0 + kb < k_end) ? B[offBk[kb] + offBn[ni]] : 0.0;
     }
 #pragma unroll
-    for (int q = 0; q < (BN * BK) / NT; ++q) {
-      int e = tid + q * NT;
-      int ni, ki;
-      if (b_kfast) { ki = e % BK; ni = e / BK; } else { ni = e % BN; ki = e / BN; }
-      int n = n0 + ni, k = k0 + ki;
-      Bs[ki][ni] = (n < g.N && k < g.K) ? B[offBk[ki] + offBn[ni]] : T(0);
+    for (int q = 0; q < 2; ++q) {
+      const int e = tid + q * NT;
+      const int mi = a_kfast ? e / BK : e % BM, ka = a_kfast ? e % BK : e / BM;
+      const int ni = b_kfast ? e / BK : e % BN, kb = b_kfast ? e % BK : e / BN;
+      As[ka][mi] = va[q];
+      Bs[kb][ni] = vb[q];
     }
     __syncthreads();
+    if (live) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[4], bb[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+      for (int kk = 0; kk < BK; ++kk) {
+        const double2 a01 = *reinterpret_cast<const double2*>(&As[kk][4 * warp]);
+        const double2 a23 = *reinterpret_cast<const double2*>(&As[kk][4 * warp + 2]);
+        const double bb = Bs[kk][lane];
+        acc[0] = fma(a01.x, bb, acc[0]);
+        acc[1] = fma(a01.y, bb, acc[1]);
+        acc[2] = fma(a23.x, bb, acc[2]);
+        acc[3] = fma(a23.y, bb, acc[3]);
+      }
     }
   }
 
-  T* C = g.C + b * g.scb;
+  double* C = g.C + b * g.scb;
+  if (!SPLIT) {
+    const int n = n0 + lane;
+    if (n >= g.N) return;
+    const long long on = off32(g.cn, n);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int m = m0 + ty + 16 * i;
-    if (m >= g.M) continue;
-    long long om = idx_off(g.cm, m);
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + 4 * warp + i;
+      if (m >= g.M) break;
+      const long long o = off32(g.cm, m) + on;
+      double v = g.alpha * acc[i];
+      if (g.beta != 0.0) v += g.beta * C[o];
+      C[o] = v;
+    }
+    return;
+  }
+  // sum of the ranks' tiles: rank r takes every splits-th row
+  __shared__ double Cs[BM][BN];
+  cg::cluster_group cluster = cg::this_cluster();
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx + 16 * j;
-      if (n >= g.N) continue;
-      long long o = om + idx_off(g.cn, n);
-      T v = (T)g.alpha * acc[i][j];
-      if (g.beta != 0.0) v += (T)g.beta * C[o];
+  for (int i = 0; i < 4; ++i) Cs[4 * warp + i][lane] = acc[i];
+  cluster.sync();
+  const int n = n0 + lane;
+  for (int row = rank + splits * warp; row < BM; row += splits * (NT / 32)) {
+    const int m = m0 + row;
+    if (m < g.M && n < g.N) {
+      double s = 0.0;
+      for (int q = 0; q < splits; ++q) s += *cluster.map_shared_rank(&Cs[row][lane], q);
+      const long long o = off32(g.cm, m) + off32(g.cn, n);
+      double v = g.alpha * s;
+      if (g.beta != 0.0) v += g.beta * C[o];
       C[o] = v;
     }
   }
+  cluster.sync();   // peers may still be reading this CTA's tile
 }
 
 int innermost_unit(const Idx3& d) {
@@ -111,19 +155,68 @@ int innermost_unit(const Idx3& d) {
   return d.s2 == 1;
 }
 
-template <typename T, typename G>
-cudaError_t launch(const G& g, cudaStream_t st) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
-  if (g.K <= 0 || g.batch > 65535) return cudaErrorInvalidValue;
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-  if (grid.y > 65535) return cudaErrorInvalidValue;
-  int a_kfast = innermost_unit(g.ak) && !innermost_unit(g.am);
-  int b_kfast = innermost_unit(g.bk) && !innermost_unit(g.bn);
-  note_launch();
-  gemm_kernel<T, G><<<grid, NT, 0, st>>>(g, a_kfast, b_kfast);
-  return cudaGetLastError();
-}
+inline long long up_to(long long x, long long q) { return (x + q - 1) / q * q; }
+
+PerDevice<int> g_sms;
 
 }  // namespace
 
-cudaError_t gemm_f64(const GemmF64& g, cudaStream_t st) { return launch<double>(g, st); }
+cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
+  if (g0.M <= 0 || g0.N <= 0 || g0.batch <= 0) return cudaSuccess;
+  if (g0.K <= 0 || g0.batch > 65535) return cudaErrorInvalidValue;
+  GemmF64 g = g0;
+  // C^T = B^T A^T when its rows and columns round up to less work
+  if (up_to(g.N, 4) * up_to(g.M, BN) < up_to(g.M, 4) * up_to(g.N, BN)) {
+    g.M = g0.N; g.N = g0.M;
+    g.A = g0.B; g.am = g0.bn; g.ak = g0.bk; g.sab = g0.sbb;
+    g.B = g0.A; g.bk = g0.ak; g.bn = g0.am; g.sbb = g0.sab;
+    g.cm = g0.cn; g.cn = g0.cm;
+  }
+  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
+  if (grid.y > 65535) return cudaErrorInvalidValue;
+  int sms = 152;
+  cudaError_t e = g_sms.get(
+      [](int dev) {
+        int n = 0;
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0
+                   ? n : 152;
+      },
+      &sms);
+  if (e != cudaSuccess) return e;
+  // Split of the contraction: the fewest K-steps on the busiest SM.  A split
+  // adds its start and the exchange of its partial tile, about two K-steps
+  // (16 x 32 x 32 FMAs at 2 a clock, 4 us each); a step is one K-block of 16.
+  const long long tiles = (long long)grid.x * grid.y * g.batch;
+  const int kb = (g.K + BK - 1) / BK;
+  int splits = 1;
+  long long best = 0;
+  for (int s = 1; s <= SPLIT_MAX && (s == 1 || (s <= kb && g.batch * s <= 65535)); s *= 2) {
+    const long long per = (kb + s - 1) / s + (s > 1 ? 2 : 0);
+    const long long cost = (tiles * s + sms - 1) / sms * per;
+    if (s == 1 || cost < best) {
+      best = cost;
+      splits = s;
+    }
+  }
+  const int a_kfast = innermost_unit(g.ak) && !innermost_unit(g.am);
+  const int b_kfast = innermost_unit(g.bk) && !innermost_unit(g.bn);
+  note_launch();
+  if (splits == 1) {
+    gemm_kernel<false><<<grid, NT, 0, st>>>(g, a_kfast, b_kfast, 1, g.K);
+    return cudaGetLastError();
+  }
+  grid.z = (unsigned)(g.batch * splits);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = (unsigned)splits;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(NT);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemm_kernel<true>, g, a_kfast, b_kfast, splits,
+                            (kb + splits - 1) / splits * BK);
+}
