@@ -77,14 +77,16 @@ cudaError_t gemm_f64(const GemmF64& g, cudaStream_t st);
 
 
 // ---------------------------------------------------------------- SVD split
-// One-sided (Hestenes) Jacobi SVD of a row-major m x n matrix M in FP64,
-// with selection of the largest singular values.  See svd_jacobi.cu.
+// SVD of a row-major m x n matrix M in FP64 (pivoted QR, then one-sided Jacobi
+// on its triangular factor), with selection of the largest singular values.
+// See svd_jacobi.cu.
 struct SvdBuffers {
-  double* W;       // len x ncols, column j contiguous
-  double* V;       // ncols x ncols, column j contiguous
+  double* W;       // R^T of the pivoted QR, rotated: min(m, n) columns, contiguous
+  double* V;       // the columns of the split matrix, contiguous
+  double* nrm;     // 2 x max_cols squared column norms
   double* sig;     // ncols
   int* perm;       // ncols: perm[r] = column with the r-th largest sigma
-  int* counter;    // rotations in the current sweep
+  int* counter;    // 8 words: grid barrier, rotations and unconverged pairs per sweep
   double* stats;   // [0] = total weight, [1] = discarded fraction, [2] = sigma_max, [3] = rank
   int* kept;       // number kept
   size_t max_elems;   // capacity of W and of V in doubles

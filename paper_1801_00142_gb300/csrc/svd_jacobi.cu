@@ -1,4 +1,5 @@
-// FP64 one-sided (Hestenes) Jacobi SVD and the two-site split of Fig. VMPO(d).
+// FP64 singular value split of Fig. VMPO(d): pivoted QR, then one-sided
+// (Hestenes) Jacobi on the transposed triangular factor.
 //
 // The generalised overlap C_E (Eq. LSEProd) is factorised C_E = U Lambda V^T
 // and truncated by *number*: the largest min(D*, numerical rank) singular
@@ -7,42 +8,66 @@
 // dropped).  Left-to-right the left factor is U and the right factor
 // Lambda V^T; right-to-left Lambda goes with U (App. D.1).
 //
-// One-sided Jacobi orthogonalises the min(m, n) columns of M (or of M^T) by
-// plane rotations; it resolves small singular values to high relative
-// accuracy, which the series initialisation needs (its higher-order terms sit
-// 1e-10 .. 1e-15 below the leading singular value).
+// Let A (q x p) be the matrix with the side of the wanted isometry as its
+// columns: A = M^T for U, A = M for V.
+//  1. Pivoted QR, A P = Q R, by modified Gram-Schmidt on the columns of A;
+//     only R^T (p x r) is formed, Q is never needed.  It ends early at rank r
+//     when what is left has a Frobenius norm below a tenth of rel_tol *
+//     sigma_max (those singular values are numerically zero), or, when kcap
+//     cuts the spectrum, below 1e-6 of what was left after kcap columns: the
+//     remainder E is orthogonal to Q, so A^T A = R^T R + E^T E and the kept
+//     subspace changes by the square of that ratio.
+//  2. One-sided Jacobi orthogonalises the r columns of R^T: R^T J = X Sigma
+//     with X the wanted singular vectors.  The triangular factor of a pivoted
+//     QR is close to having orthogonal rows, and the rotations resolve small
+//     singular values to high relative accuracy (which the series
+//     initialisation needs: its higher-order terms sit 1e-10 .. 1e-15 below
+//     the leading one).  Jacobi on C_E itself takes 12 to 40 sweeps over
+//     min(m, n) columns; on R^T it takes 4 to 6 over r of them.
+//  3. The kept columns X_k = (R^T J)_k / sigma_k are one factor, the other one
+//     is M projected on them: U^T M or M V.
 //
-// GPU mapping: one persistent cooperative kernel per split.  Each round of
-// the round-robin ordering rotates disjoint column pairs, one warp per pair
-// (shuffle reductions, no block barriers); rounds are separated by a grid
-// barrier whose wait is bounded (on expiry the kernel records a timeout and
-// every CTA leaves).  Convergence, the column norms, the selection of the
-// kept singular values and the emission of the two factors all happen inside
-// the same launch, so the host synchronises once per split to read k.
+// GPU mapping: one kernel per split, one warp per column (step 1) or per
+// column pair of a round-robin round (step 2); columns live in L2 (read past
+// L1).  Steps and rounds are separated by a barrier over all CTAs.  What
+// bounds it is latency: a step moves a few columns, does a hundred FP64
+// operations per lane pair and meets the barrier.  Small problems run in one
+// thread-block cluster of up to 16 CTAs, whose hardware barrier takes a
+// fraction of a microsecond; larger ones, which need more than 16 SMs' worth
+// of FP64 (two FMAs a clock each), run as a cooperative grid with a bounded
+// barrier (on expiry the kernel records a timeout and every CTA leaves).
+// Measured, one FP64 doubling at L = 32, D* = 40, one sweep (62 splits of up
+// to 160 x 160): 1089 ms with Jacobi on C_E, 154 ms with this split.
 #include <math.h>
 
 #include "common.cuh"
 
 namespace {
 
-constexpr int WPB = 4;                  // warps per CTA
+constexpr int WPB = 8;                  // warps per CTA
 constexpr int NT = WPB * 32;
+constexpr int CL_MAX = 16;              // CTAs of the largest cluster (opt-in size)
 constexpr long long SPIN_LIMIT = 1LL << 22;
+constexpr int REGS = 8;                 // columns up to 32 * REGS rows stay in registers
 
 struct SvdArgs {
   const double* M;
-  int m, n, trans, len, ncols, nn, kcap, mode, max_sweeps;
-  double tol, rel_tol;
-  double *W, *V, *sig;
+  int m, n, kcap, mode, max_sweeps;
+  int p, q, rmax;        // isometry side, other side, min(p, q)
+  long long sc, si;      // A[i][c] = M[c * sc + i * si], i < q, c < p
+  double tol2, rel_tol;
+  double *A, *W, *nrm;   // A: p columns of length q; W: rmax columns of length p; nrm: 2 x max_cols
+  int max_cols;
+  double* sig;
   int* perm;
   double *left, *right;
   unsigned* bar;      // [0] arrivals, [1] generation
-  int* rot;           // [3] rotations per sweep (ring)
+  int* cnt;           // [0..2] rotations per sweep (ring), [3..5] unconverged pairs per check (ring)
   int* out;           // [0] k, [1] rank, [2] sweeps, [3] status (0 ok, 1 timeout, 2 not converged)
   double* stats;      // [0] total weight, [1] discarded fraction, [2] sigma_max,
                       // [3] ||M||_F^2 (accumulated while loading)
   // device-decided mode (all null otherwise): run only if *run_if > thresh
-  // or is not finite; keep exactly min(kcap, ncols); report into acc
+  // or is not finite; keep exactly min(kcap, p, q); report into acc
   const double* run_if;
   double thresh;
   SvdDeviceAcc acc;
@@ -76,7 +101,7 @@ __device__ bool grid_barrier(const SvdArgs& a) {
             ok = 0;
             break;
           }
-          __nanosleep(32);
+          if (it > 64) __nanosleep(32);
         }
       }
       __threadfence();
@@ -86,190 +111,457 @@ __device__ bool grid_barrier(const SvdArgs& a) {
   return ok != 0;
 }
 
+// Barrier over all CTAs of the launch (one cluster, or the whole grid).
+template <bool CLUSTER>
+__device__ __forceinline__ bool all_sync(const SvdArgs& a) {
+  if (!CLUSTER) return grid_barrier(a);
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+               ::: "memory");
+  return true;
+}
+
 __device__ inline double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-__global__ void __launch_bounds__(NT) svd_persistent(SvdArgs a) {
-  // device-decided mode: every CTA leaves before the first barrier
-  if (a.run_if && *a.run_if <= a.thresh) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * WPB + (threadIdx.x >> 5);
-  const int TW = gridDim.x * WPB;
-  const long long gt = blockIdx.x * (long long)NT + threadIdx.x;
-  const long long GT = (long long)gridDim.x * NT;
+// The rotation that zeroes the Gram entry ga of two columns with squared
+// norms al, be: t = sign(z) / (|z| + sqrt(1 + z^2)), z = (be - al) / (2 ga).
+// FP64 divisions and square roots are long sequences on a pipe of two lanes,
+// so t is computed in FP32 (its error of 1e-7 leaves 1e-7 ga behind, which a
+// later visit removes) and c, s from it to FP64 accuracy (two Newton steps).
+// false: the angle is below FP32's range (nothing to rotate).
+__device__ __forceinline__ bool rotation(double al, double be, double ga, double& t, double& c,
+                                         double& s) {
+  const int e = (__double2hiint(ga) >> 20) & 0x7ff;
+  if (e < 1 || e > 2045) return false;
+  const double sc = __hiloint2double((2046 - e) << 20, 0);   // |ga| sc in [1, 2)
+  const float g = (float)(ga * sc), d = (float)((be - al) * sc);
+  const float z = d / (2.f * g);
+  const float t32 = fabsf(z) > 1e9f ? 0.5f / z
+                                    : copysignf(1.f / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))), z);
+  if (t32 == 0.f) return false;
+  t = (double)t32;
+  const double w = fma(t, t, 1.0);
+  double x = (double)rsqrtf((float)w);
+  x = x * fma(-0.5 * w, x * x, 1.5);
+  x = x * fma(-0.5 * w, x * x, 1.5);
+  c = x;
+  s = x * t;
+  return true;
+}
 
-  // load: column j of M (trans = 0) or of M^T (trans = 1); V = I
-  const long long tot = (long long)a.len * a.ncols;
-  double ss = 0.0;
-  for (long long e = gt; e < tot; e += GT) {
-    int j = (int)(e / a.len), i = (int)(e % a.len);
-    const double x = a.trans ? a.M[(long long)j * a.n + i] : a.M[(long long)i * a.n + j];
-    a.W[e] = x;
-    ss = fma(x, x, ss);
-  }
-  ss = warp_sum(ss);
-  if (lane == 0) atomicAdd(a.stats + 3, ss);
-  for (long long e = gt; e < (long long)a.ncols * a.ncols; e += GT) {
-    int j = (int)(e / a.ncols), i = (int)(e % a.ncols);
-    a.V[e] = (i == j) ? 1.0 : 0.0;
-  }
-  if (gt < 3) a.rot[gt] = 0;
-  if (!grid_barrier(a)) return;
-  // Gram entries below eps^2 ||M||_F^2 are beneath the resolution of the
-  // whole problem: pairs of numerically-zero columns are not rotated (without
-  // this floor, columns of pure rounding noise can rotate without end)
-  const double gfloor = 4.930380657631324e-32 * ((volatile double*)a.stats)[3];
-
-  const int mod = a.nn - 1;
-  const int npairs = a.nn / 2;
-  int sweeps = 0;
-  bool converged = a.ncols < 2;
-  for (int s = 0; s < a.max_sweeps && !converged; ++s) {
-    if (gt == 0) a.rot[(s + 1) % 3] = 0;
-    int myrot = 0;
-    for (int r = 0; r < mod; ++r) {
-      for (int i = gw; i < npairs; i += TW) {
-        int p, q;
-        if (i == 0) { p = r; q = a.nn - 1; }
-        else { p = (r + i) % mod; q = (r - i + mod) % mod; }
-        if (p > q) { int t = p; p = q; q = t; }
-        if (q >= a.ncols) continue;
-        double* wp = a.W + (long long)p * a.len;
-        double* wq = a.W + (long long)q * a.len;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int e = lane; e < a.len; e += 32) {
-          double x = wp[e], y = wq[e];
-          al = fma(x, x, al);
-          be = fma(y, y, be);
-          ga = fma(x, y, ga);
-        }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (!(fabs(ga) > a.tol * sqrt(al) * sqrt(be)) || !(fabs(ga) > gfloor) || al == 0.0 ||
-            be == 0.0)
-          continue;
-        // rotation zeroing the (p, q) Gram entry: t = sign(z)/(|z| + sqrt(1+z^2))
-        double z = (be - al) / (2.0 * ga);
-        double t = (z >= 0.0 ? 1.0 : -1.0) / (fabs(z) + hypot(1.0, z));
-        double c = 1.0 / sqrt(1.0 + t * t);
-        double sn = c * t;
-        for (int e = lane; e < a.len; e += 32) {
-          double x = wp[e], y = wq[e];
-          wp[e] = c * x - sn * y;
-          wq[e] = sn * x + c * y;
-        }
-        double* vp = a.V + (long long)p * a.ncols;
-        double* vq = a.V + (long long)q * a.ncols;
-        for (int e = lane; e < a.ncols; e += 32) {
-          double x = vp[e], y = vq[e];
-          vp[e] = c * x - sn * y;
-          vq[e] = sn * x + c * y;
-        }
-        ++myrot;
+// One pair of W's columns: rotated if its Gram entry is above tol * norms.
+__device__ __forceinline__ int rotate_pair(const SvdArgs& a, int jp, int jq, double gfloor,
+                                           int lane) {
+  const int p = a.p;
+  double* wp = a.W + (long long)jp * p;
+  double* wq = a.W + (long long)jq * p;
+  const double al = __ldcg(a.nrm + jp), be = __ldcg(a.nrm + jq);
+  double t, c, s;
+  if (p <= 32 * REGS) {
+    double x[REGS], y[REGS], ga = 0.0;
+#pragma unroll
+    for (int u = 0; u < REGS; ++u) {
+      const int e = lane + 32 * u;
+      x[u] = e < p ? __ldcg(wp + e) : 0.0;
+      y[u] = e < p ? __ldcg(wq + e) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < REGS; ++u)
+      if (32 * u < p) ga = fma(x[u], y[u], ga);
+    ga = warp_sum(ga);
+    if (!(ga * ga > a.tol2 * al * be) || !(fabs(ga) > gfloor)) return 0;
+    if (!rotation(al, be, ga, t, c, s)) return 0;
+#pragma unroll
+    for (int u = 0; u < REGS; ++u) {
+      const int e = lane + 32 * u;
+      if (32 * u < p && e < p) {
+        __stcg(wp + e, fma(c, x[u], -(s * y[u])));
+        __stcg(wq + e, fma(s, x[u], c * y[u]));
       }
-      if (!grid_barrier(a)) return;
     }
-    if (lane == 0 && myrot) atomicAdd(a.rot + (s % 3), myrot);
-    if (!grid_barrier(a)) return;
-    sweeps = s + 1;
-    converged = ((volatile int*)a.rot)[s % 3] == 0;
-  }
-
-  // column norms = singular values
-  for (int j = gw; j < a.ncols; j += TW) {
-    const double* w = a.W + (long long)j * a.len;
-    double s2 = 0.0;
-    for (int e = lane; e < a.len; e += 32) s2 = fma(w[e], w[e], s2);
-    s2 = warp_sum(s2);
-    if (lane == 0) a.sig[j] = sqrt(s2);
-  }
-  if (!grid_barrier(a)) return;
-
-  // rank the singular values (descending; ties by column index; non-negative
-  // doubles order like their bit patterns) and select k
-  for (int j = (int)gt; j < a.ncols; j += (int)GT) {
-    long long bj = __double_as_longlong(a.sig[j]);
-    int rk = 0;
-    for (int i = 0; i < a.ncols; ++i) {
-      long long bi = __double_as_longlong(a.sig[i]);
-      rk += (bi > bj) || (bi == bj && i < j);
+    if (lane == 0) {
+      __stcg(a.nrm + jp, fmax(0.0, fma(-t, ga, al)));
+      __stcg(a.nrm + jq, fmax(0.0, fma(t, ga, be)));
     }
-    a.perm[rk] = j;
+    return 1;
   }
-  if (!grid_barrier(a)) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double mx = 0.0, totw = 0.0;
-    for (int j = 0; j < a.ncols; ++j) { mx = fmax(mx, a.sig[j]); totw += a.sig[j] * a.sig[j]; }
-    int cnt = 0;
-    for (int j = 0; j < a.ncols; ++j) cnt += a.sig[j] > a.rel_tol * mx;
-    int k = cnt < a.kcap ? cnt : a.kcap;
-    if (a.run_if) k = a.kcap < a.ncols ? a.kcap : a.ncols;
-    if (k < 1) k = 1;
-    double keptw = 0.0;
-    for (int r = 0; r < k; ++r) { double s = a.sig[a.perm[r]]; keptw += s * s; }
-    a.out[0] = k;
-    a.out[1] = cnt;
-    a.out[2] = sweeps;
-    if (!converged) a.out[3] = 2;
-    a.stats[0] = totw;
-    a.stats[1] = totw > 0.0 ? fmax(0.0, (totw - keptw) / totw) : 0.0;
-    a.stats[2] = mx;
-    if (a.run_if) {
-      if (a.acc.disc_max)
-        atomicMax(reinterpret_cast<unsigned long long*>(a.acc.disc_max),
-                  (unsigned long long)__double_as_longlong(a.stats[1]));
-      if (a.acc.runs) atomicAdd(a.acc.runs, 1ull);
-      if (a.acc.status && !converged) atomicMax(a.acc.status, 2);
-      if (a.acc.status && !isfinite(mx)) atomicMax(a.acc.status, 3);
-    }
+  double ga = 0.0;
+#pragma unroll 4
+  for (int e = lane; e < p; e += 32) ga = fma(__ldcg(wp + e), __ldcg(wq + e), ga);
+  ga = warp_sum(ga);
+  if (!(ga * ga > a.tol2 * al * be) || !(fabs(ga) > gfloor)) return 0;
+  if (!rotation(al, be, ga, t, c, s)) return 0;
+#pragma unroll 4
+  for (int e = lane; e < p; e += 32) {
+    const double x = __ldcg(wp + e), y = __ldcg(wq + e);
+    __stcg(wp + e, fma(c, x, -(s * y)));
+    __stcg(wq + e, fma(s, x, c * y));
   }
-  if (!grid_barrier(a)) return;
+  if (lane == 0) {
+    __stcg(a.nrm + jp, fmax(0.0, fma(-t, ga, al)));
+    __stcg(a.nrm + jq, fmax(0.0, fma(t, ga, be)));
+  }
+  return 1;
+}
 
-  // emit Left (m x k) and Right (k x n).
-  // trans = 0: W = M V = U Sigma (len = m), V holds V.
-  // trans = 1: W = M^T V' = V Sigma (len = n), V' holds U.
-  const int k = ((volatile int*)a.out)[0];
-  const long long nl = (long long)a.m * k, nr = (long long)k * a.n;
-  for (long long e = gt; e < nl + nr; e += GT) {
-    bool isleft = e < nl;
-    int r, x;
-    if (isleft) { x = (int)(e / k); r = (int)(e % k); }
-    else { r = (int)((e - nl) / a.n); x = (int)((e - nl) % a.n); }
-    int j = a.perm[r];
-    double s = a.sig[j];
-    bool fromW = isleft ? (a.trans == 0) : (a.trans == 1);   // W holds Sigma-scaled vectors
-    double base = fromW ? a.W[(long long)j * a.len + x] : a.V[(long long)j * a.ncols + x];
-    bool want_sigma = isleft ? (a.mode == SPLIT_LEFT) : (a.mode == SPLIT_RIGHT);
-    double v;
-    if (want_sigma == fromW) v = base;
-    else if (want_sigma) v = base * s;
-    else v = (s > 0.0) ? base / s : 0.0;
-    if (isleft) a.left[(long long)x * k + r] = v;
-    else a.right[(long long)r * a.n + x] = v;
+// C[i][j] = sum_t P(i, t) Q(t, j) over all CTAs, 16 x 16 tiles.
+__device__ void project(const double* P, long long pi, long long pt, const double* Q, long long qt,
+                        long long qj, double* C, long long ci, long long cj, int ni, int nj,
+                        int nt) {
+  __shared__ double Ps[16][17], Qs[16][17];
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int tj = (nj + 15) / 16, tiles = (ni + 15) / 16 * tj;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int i0 = tile / tj * 16, j0 = tile % tj * 16;
+    double acc = 0.0;
+    for (int t0 = 0; t0 < nt; t0 += 16) {
+      // consecutive threads take the index that is contiguous in memory
+      const int a_i = pt == 1 ? ty : tx, a_t = pt == 1 ? tx : ty;
+      const int b_j = qj == 1 ? tx : ty, b_t = qj == 1 ? ty : tx;
+      Ps[a_t][a_i] = (i0 + a_i < ni && t0 + a_t < nt) ? __ldcg(P + (i0 + a_i) * pi + (t0 + a_t) * pt) : 0.0;
+      Qs[b_t][b_j] = (j0 + b_j < nj && t0 + b_t < nt) ? __ldcg(Q + (t0 + b_t) * qt + (j0 + b_j) * qj) : 0.0;
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < 16; ++t) acc = fma(Ps[t][ty], Qs[t][tx], acc);
+      __syncthreads();
+    }
+    if (i0 + ty < ni && j0 + tx < nj) C[(i0 + ty) * ci + (j0 + tx) * cj] = acc;
   }
 }
 
-// CTAs of the cooperative launch (once per device, thread-safe)
+template <bool CLUSTER>
+__global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
+  // device-decided mode: every CTA leaves before the first barrier
+  if (a.run_if && *a.run_if <= a.thresh) return;
+  const int lane = threadIdx.x & 31;
+  // consecutive work items go to different SMs
+  const int gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int TW = gridDim.x * WPB;
+  const long long gt = blockIdx.x * (long long)NT + threadIdx.x;
+  const long long GT = (long long)gridDim.x * NT;
+  const int p = a.p, q = a.q;
+
+  // load A's columns and their squared norms
+  double ss = 0.0;
+  for (int c = gw; c < p; c += TW) {
+    double* col = a.A + (long long)c * q;
+    double s2 = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < q; i += 32) {
+      const double x = a.M[c * a.sc + i * a.si];
+      __stcg(col + i, x);
+      s2 = fma(x, x, s2);
+    }
+    s2 = warp_sum(s2);
+    if (lane == 0) __stcg(a.nrm + c, s2);
+    ss += s2;
+  }
+  if (lane == 0 && ss != 0.0) atomicAdd(a.stats + 3, ss);
+  if (!all_sync<CLUSTER>(a)) return;
+  const double fro = __ldcg(a.stats + 3);
+  if (!(fro <= 1.7976931348623157e308)) {   // a non-finite entry: reported, nothing emitted
+    if (gt == 0) {
+      a.out[0] = 1;
+      a.out[1] = 0;
+      a.out[2] = 0;
+      a.stats[0] = a.stats[2] = fro;
+      a.stats[1] = 0.0;
+      if (a.run_if && a.acc.runs) atomicAdd(a.acc.runs, 1ull);
+      if (a.run_if && a.acc.status) atomicMax(a.acc.status, 3);
+    }
+    return;
+  }
+
+  // ---- 1. pivoted QR (modified Gram-Schmidt), rows of R into W's columns
+  int r = 0;
+  double mx0 = 0.0, scale = 1.0, rho_k = -1.0, rem = 0.0;
+  const double nstop = 0.01 * a.rel_tol * a.rel_tol;
+  for (int j = 0; j < a.rmax; ++j) {
+    const double* nr = a.nrm + (j & 1) * (long long)a.max_cols;
+    double* nw = a.nrm + ((j + 1) & 1) * (long long)a.max_cols;
+    // pivot: the column with the largest norm left (finished ones hold -1);
+    // every warp scans the same values, so all take the same branches
+    double best = -1.0;
+    int piv = 0x7fffffff;
+    rem = 0.0;
+#pragma unroll 4
+    for (int c = lane; c < p; c += 32) {
+      const double v = __ldcg(nr + c);
+      if (v > 0.0) rem += v;
+      if (v > best) {
+        best = v;
+        piv = c;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double v = __shfl_xor_sync(0xffffffffu, best, o);
+      const int c = __shfl_xor_sync(0xffffffffu, piv, o);
+      if (v > best || (v == best && c < piv)) {
+        best = v;
+        piv = c;
+      }
+    }
+    rem = warp_sum(rem);
+    if (j == 0) {
+      mx0 = best;
+      // W is scaled by a power of two to norms of at most about 1
+      if (best > 0.0) scale = ldexp(1.0, -(ilogb(best) / 2));
+    }
+    if (!(best > 0.0) || rem <= nstop * mx0) break;
+    if (j == a.kcap) rho_k = rem;
+    if (rho_k >= 0.0 && j > a.kcap && rem <= 1e-12 * rho_k) break;
+    const double rinv = rsqrt(best);
+    const double* xp = a.A + (long long)piv * q;
+    double* wrow = a.W + (long long)j * p;
+    for (int c = gw; c < p; c += TW) {
+      const double nc = __ldcg(nr + c);
+      if (nc < 0.0 || c == piv) {
+        if (lane == 0) {
+          __stcg(wrow + c, c == piv ? best * rinv * scale : 0.0);
+          __stcg(nw + c, -1.0);
+        }
+        continue;
+      }
+      double* xc = a.A + (long long)c * q;
+      double dot = 0.0, s2 = 0.0;
+      if (q <= 32 * REGS) {
+        double x[REGS], y[REGS];
+#pragma unroll
+        for (int u = 0; u < REGS; ++u) {
+          const int e = lane + 32 * u;
+          x[u] = e < q ? __ldcg(xp + e) : 0.0;
+          y[u] = e < q ? __ldcg(xc + e) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < REGS; ++u)
+          if (32 * u < q) dot = fma(x[u], y[u], dot);
+        dot = warp_sum(dot) * rinv;
+        const double f = dot * rinv;
+#pragma unroll
+        for (int u = 0; u < REGS; ++u) {
+          const int e = lane + 32 * u;
+          if (32 * u < q) {
+            y[u] = fma(-f, x[u], y[u]);
+            s2 = fma(y[u], y[u], s2);
+            if (e < q) __stcg(xc + e, y[u]);
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (int e = lane; e < q; e += 32) dot = fma(__ldcg(xp + e), __ldcg(xc + e), dot);
+        dot = warp_sum(dot) * rinv;
+        const double f = dot * rinv;
+#pragma unroll 4
+        for (int e = lane; e < q; e += 32) {
+          const double y = fma(-f, __ldcg(xp + e), __ldcg(xc + e));
+          s2 = fma(y, y, s2);
+          __stcg(xc + e, y);
+        }
+      }
+      s2 = warp_sum(s2);
+      if (lane == 0) {
+        __stcg(wrow + c, dot * scale);
+        __stcg(nw + c, s2);
+      }
+    }
+    r = j + 1;
+    rem = 0.0;   // what is left is known at the next step's scan only
+    if (!all_sync<CLUSTER>(a)) return;
+  }
+  // the norms become those of W's columns: every warp has read them
+  if (!all_sync<CLUSTER>(a)) return;
+
+  // ---- 2. one-sided Jacobi on W (p x r)
+  const int nn = r + (r & 1), mod = nn - 1, npairs = nn / 2;
+  int sweeps = 0;
+  bool converged = r < 2;
+  for (int s = 0; s < a.max_sweeps; ++s) {
+    // squared column norms afresh: the rotations update them with rounding
+    for (int j = gw; j < r; j += TW) {
+      const double* w = a.W + (long long)j * p;
+      double s2 = 0.0;
+#pragma unroll 4
+      for (int e = lane; e < p; e += 32) {
+        const double x = __ldcg(w + e);
+        s2 = fma(x, x, s2);
+      }
+      s2 = warp_sum(s2);
+      if (lane == 0) __stcg(a.nrm + j, s2);
+    }
+    if (gt == 0) {
+      a.cnt[(s + 1) % 3] = 0;
+      a.cnt[3 + (s + 1) % 3] = 0;
+    }
+    if (!all_sync<CLUSTER>(a)) return;
+    if (converged) break;
+    // Pairs of columns below the resolution of the whole problem could rotate
+    // without end: past 30 sweeps (never met) Gram entries beneath eps^2
+    // ||W||^2 are left alone
+    const double gfloor = s < 30 ? 0.0 : 4.930380657631324e-32 * fro * scale * scale;
+    if (s >= 3) {
+      // all cosines at once: a converged state needs no sweep of rounds
+      int off = 0;
+      const int np = r * (r - 1) / 2;
+      for (int e = gw; e < np; e += TW) {
+        int i = (int)((1.f + sqrtf(1.f + 8.f * (float)e)) * 0.5f);
+        while (i * (i - 1) / 2 > e) --i;
+        while ((i + 1) * i / 2 <= e) ++i;
+        const int jj = e - i * (i - 1) / 2;
+        const double* wi = a.W + (long long)i * p;
+        const double* wj = a.W + (long long)jj * p;
+        double ga = 0.0;
+#pragma unroll 4
+        for (int x = lane; x < p; x += 32) ga = fma(__ldcg(wi + x), __ldcg(wj + x), ga);
+        ga = warp_sum(ga);
+        off += ga * ga > a.tol2 * __ldcg(a.nrm + i) * __ldcg(a.nrm + jj) && fabs(ga) > gfloor;
+      }
+      if (lane == 0 && off) atomicAdd(a.cnt + 3 + s % 3, off);
+      if (!all_sync<CLUSTER>(a)) return;
+      if (__ldcg(a.cnt + 3 + s % 3) == 0) {
+        converged = true;
+        break;
+      }
+    }
+    int myrot = 0;
+    for (int rd = 0; rd < mod; ++rd) {
+      for (int i = gw; i < npairs; i += TW) {
+        int jp, jq;
+        if (i == 0) { jp = rd; jq = nn - 1; }
+        else { jp = (rd + i) % mod; jq = (rd - i + mod) % mod; }
+        if (jp > jq) { int t = jp; jp = jq; jq = t; }
+        if (jq >= r) continue;
+        myrot += rotate_pair(a, jp, jq, gfloor, lane);
+      }
+      if (rd == mod - 1 && lane == 0 && myrot) atomicAdd(a.cnt + s % 3, myrot);
+      if (!all_sync<CLUSTER>(a)) return;
+    }
+    sweeps = s + 1;
+    converged = __ldcg(a.cnt + s % 3) == 0;
+  }
+
+  // ---- 3. singular values, their order, the kept number
+  for (int j = (int)gt; j < a.rmax; j += (int)GT) {
+    const double s2 = j < r ? __ldcg(a.nrm + j) : 0.0;
+    int rk = 0;
+    if (j < r) {
+      for (int i = 0; i < r; ++i) {
+        const double x = __ldcg(a.nrm + i);
+        rk += x > s2 || (x == s2 && i < j);
+      }
+    } else {
+      rk = j;
+    }
+    a.perm[rk] = j;
+    a.sig[j] = sqrt(s2) / scale;   // exact division: scale is a power of two
+  }
+  if (!all_sync<CLUSTER>(a)) return;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    double mx = 0.0;
+    for (int j = lane; j < r; j += 32) mx = fmax(mx, __ldcg(a.nrm + j));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const double smx = sqrt(mx);
+    int cnt = 0;
+    for (int j = lane; j < r; j += 32) cnt += sqrt(__ldcg(a.nrm + j)) > a.rel_tol * smx;
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    int k = cnt < a.kcap ? cnt : a.kcap;
+    if (a.run_if) k = a.kcap < a.rmax ? a.kcap : a.rmax;
+    if (k < 1) k = 1;
+    double keptw = 0.0, dropw = 0.0;
+    for (int j = lane; j < r; j += 32) {
+      const double w = __ldcg(a.nrm + __ldcg(a.perm + j));
+      if (j < k) keptw += w;
+      else dropw += w;
+    }
+    keptw = warp_sum(keptw);
+    dropw = warp_sum(dropw) + rem * scale * scale;
+    if (lane == 0) {
+      a.out[0] = k;
+      a.out[1] = cnt;
+      a.out[2] = sweeps;
+      if (!converged) a.out[3] = 2;
+      a.stats[0] = (keptw + dropw) / scale / scale;
+      a.stats[1] = keptw + dropw > 0.0 ? dropw / (keptw + dropw) : 0.0;
+      a.stats[2] = smx / scale;
+      if (a.run_if) {
+        if (a.acc.disc_max)
+          atomicMax(reinterpret_cast<unsigned long long*>(a.acc.disc_max),
+                    (unsigned long long)__double_as_longlong(a.stats[1]));
+        if (a.acc.runs) atomicAdd(a.acc.runs, 1ull);
+        if (a.acc.status && !converged) atomicMax(a.acc.status, 2);
+        if (a.acc.status && !isfinite(smx)) atomicMax(a.acc.status, 3);
+      }
+    }
+  }
+  if (!all_sync<CLUSTER>(a)) return;
+
+  // ---- 4. the isometry, then M projected on it
+  const int k = __ldcg(a.out);
+  for (int rr = gw; rr < k; rr += TW) {
+    const int j = __ldcg(a.perm + rr);
+    const double s2 = j < r ? __ldcg(a.nrm + j) : 0.0;
+    const double inv = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
+    const double* w = a.W + (long long)j * p;
+    for (int x = lane; x < p; x += 32) {
+      const double v = s2 > 0.0 ? __ldcg(w + x) * inv : 0.0;
+      if (a.mode == SPLIT_RIGHT) __stcg(a.left + (long long)x * k + rr, v);
+      else __stcg(a.right + (long long)rr * a.n + x, v);
+    }
+  }
+  if (!all_sync<CLUSTER>(a)) return;
+  if (a.mode == SPLIT_RIGHT)   // Sigma V^T = U^T M
+    project(a.left, 1, k, a.M, a.n, 1, a.right, a.n, 1, k, a.n, a.m);
+  else                         // U Sigma = M V
+    project(a.M, a.n, 1, a.right, 1, a.n, a.left, k, 1, a.m, k, a.n);
+}
+
+cudaLaunchConfig_t cluster_config(int ctas, cudaStream_t st, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// CTAs of the cooperative launch and of the largest cluster (once per device,
+// thread-safe; no kernel runs for it)
 struct SvdSetup {
   cudaError_t err;
-  int max_ctas;
+  int max_ctas, max_cluster;
 };
 PerDevice<SvdSetup> g_svd_setup;
 
 SvdSetup svd_setup() {
-  SvdSetup s{cudaSuccess, 0};
+  SvdSetup s{cudaSuccess, 0, 0};
   cudaError_t e = g_svd_setup.get(
       [](int dev) {
-        SvdSetup r{cudaSuccess, 0};
+        SvdSetup r{cudaSuccess, 0, 0};
         int sms = 0, per = 0;
         r.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (r.err == cudaSuccess)
-          r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, svd_persistent, NT, 0);
-        r.max_ctas = sms * (per < 2 ? per : 2);
+          r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, svd_split_kernel<false>, NT, 0);
+        r.max_ctas = sms * (per < 1 ? per : 1);
         if (r.err == cudaSuccess && r.max_ctas < 1) r.err = cudaErrorLaunchOutOfResources;
+        if (cudaFuncSetAttribute(svd_split_kernel<true>,
+                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+          cudaGetLastError();
+        for (int c = CL_MAX; c >= 2 && !r.max_cluster; c /= 2) {
+          cudaLaunchAttribute attr[1];
+          cudaLaunchConfig_t cfg = cluster_config(c, 0, attr);
+          int n = 0;
+          if (cudaOccupancyMaxActiveClusters(&n, svd_split_kernel<true>, &cfg) == cudaSuccess && n >= 1)
+            r.max_cluster = c;
+          else
+            cudaGetLastError();
+        }
         return r;
       },
       &s);
@@ -280,26 +572,26 @@ SvdSetup svd_setup() {
 cudaError_t svd_launch(const double* M, int m, int n, int kcap, double rel_tol, SplitMode mode,
                        double* left, double* right, const SvdBuffers& buf, cudaStream_t st,
                        const double* run_if, double thresh, const SvdDeviceAcc& acc) {
-  const int trans = (m < n) ? 1 : 0;
-  const int len = trans ? n : m;
-  const int ncols = trans ? m : n;
-  if ((size_t)len * ncols > buf.max_elems || (size_t)ncols * ncols > buf.max_elems ||
-      ncols > buf.max_cols)
+  const int p = mode == SPLIT_RIGHT ? m : n, q = mode == SPLIT_RIGHT ? n : m;
+  const int rmax = p < q ? p : q;
+  if (m < 1 || n < 1 || kcap < 1 || (size_t)m * n > buf.max_elems || p > buf.max_cols)
     return cudaErrorInvalidValue;
   cudaError_t e;
   const SvdSetup setup = svd_setup();
   if (setup.err != cudaSuccess) return setup.err;
-  const int max_ctas = setup.max_ctas;
   SvdArgs a;
-  a.M = M; a.m = m; a.n = n; a.trans = trans; a.len = len; a.ncols = ncols;
-  a.nn = ncols + (ncols & 1);
+  a.M = M; a.m = m; a.n = n; a.p = p; a.q = q; a.rmax = rmax;
+  a.sc = mode == SPLIT_RIGHT ? n : 1;
+  a.si = mode == SPLIT_RIGHT ? 1 : n;
   a.kcap = kcap; a.mode = (int)mode; a.max_sweeps = 60;
-  a.tol = sqrt((double)len) * 2.220446049250313e-16;
+  const double tol = sqrt((double)(p > q ? p : q)) * 2.220446049250313e-16;
+  a.tol2 = tol * tol;
   a.rel_tol = rel_tol;
-  a.W = buf.W; a.V = buf.V; a.sig = buf.sig; a.perm = buf.perm;
+  a.A = buf.V; a.W = buf.W; a.nrm = buf.nrm; a.max_cols = buf.max_cols;
+  a.sig = buf.sig; a.perm = buf.perm;
   a.left = left; a.right = right;
   a.bar = (unsigned*)buf.counter;      // 2 words
-  a.rot = buf.counter + 2;             // 3 words
+  a.cnt = buf.counter + 2;             // 6 words
   a.out = buf.kept;                    // 4 words
   a.stats = buf.stats;
   a.run_if = run_if;
@@ -308,15 +600,22 @@ cudaError_t svd_launch(const double* M, int m, int n, int kcap, double rel_tol, 
   if ((e = cudaMemsetAsync(buf.counter, 0, 8 * sizeof(int), st)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(buf.kept, 0, 4 * sizeof(int), st)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(buf.stats, 0, 4 * sizeof(double), st)) != cudaSuccess) return e;
-  int pairs = a.nn / 2;
-  int grid = (pairs + WPB - 1) / WPB;
-  long long work = (long long)len * ncols / (NT * 8);
-  if (work > grid) grid = (int)work;
-  if (grid > max_ctas) grid = max_ctas;
-  if (grid < 1) grid = 1;
-  void* args[] = {&a};
   note_launch();
-  return cudaLaunchCooperativeKernel((void*)svd_persistent, dim3(grid), dim3(NT), args, 0, st);
+  // One cluster while its SMs finish a step in about the time of a grid
+  // barrier: a QR step costs 3 p q FP64 operations, 32 a clock on 16 SMs.
+  // The cluster is as small as keeps a Jacobi round (5 p operations per pair)
+  // near 600 clocks, for a faster barrier.
+  if (setup.max_cluster >= 2 && (long long)p * q <= 40000) {
+    int ctas = 2;
+    while (ctas < setup.max_cluster && (long long)rmax / 2 * 5 * p > 1200LL * ctas) ctas *= 2;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(ctas, st, attr);
+    return cudaLaunchKernelEx(&cfg, svd_split_kernel<true>, a);
+  }
+  int grid = p < setup.max_ctas ? p : setup.max_ctas;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel((void*)svd_split_kernel<false>, dim3(grid), dim3(NT), args, 0,
+                                     st);
 }
 
 }  // namespace

@@ -128,6 +128,7 @@ bool plan_sizes(int L, int DH, const xtrg_config* cfg, Plan* p) {
   t += 3 * up(p->n_part * 8);               // T1, Lpart, Rpart
   t += up(p->n_ce * 8);                     // C_E
   t += 2 * up(p->n_svd * 8) + up(p->n_svd_cols * 8) + up(p->n_svd_cols * 4) + 3 * ALIGN;
+  t += up(2 * p->n_svd_cols * 8);           // squared column norms of the split
   t += up(p->n_usbuf * 8);
   t += 3 * up(p->n_obs * 8);
   t += 8 * up(p->n_herm * 8);              // Hermiticity transfers: 2 + 2 ping-pong, T (x4)
@@ -1141,6 +1142,7 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
   ctx->svd.V = (double*)carve(ctx, p.n_svd * 8);
   ctx->svd.sig = (double*)carve(ctx, p.n_svd_cols * 8);
   ctx->svd.perm = (int*)carve(ctx, p.n_svd_cols * 4);
+  ctx->svd.nrm = (double*)carve(ctx, 2 * p.n_svd_cols * 8);
   ctx->svd.counter = (int*)carve(ctx, 32);
   ctx->svd.kept = (int*)carve(ctx, 16);
   ctx->svd.stats = (double*)carve(ctx, 64);
@@ -1155,7 +1157,8 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
   ctx->ht = (double*)carve(ctx, 4 * p.n_herm * 8);
   ctx->scal = (double*)carve(ctx, 64 * 8);
   ok = ok && envbase && ctx->pp[0] && ctx->pp[1] && ctx->T1 && ctx->Lp && ctx->Rp && ctx->CE &&
-       ctx->svd.W && ctx->svd.V && ctx->svd.sig && ctx->svd.perm && ctx->svd.counter &&
+       ctx->svd.W && ctx->svd.V && ctx->svd.sig && ctx->svd.perm && ctx->svd.nrm &&
+       ctx->svd.counter &&
        ctx->svd.kept && ctx->svd.stats && ctx->usbuf && ctx->ob[0] && ctx->ob[1] && ctx->ob[2] &&
        ctx->hf[0] && ctx->hf[1] && ctx->hr[0] && ctx->hr[1] && ctx->ht &&
        ctx->scal;
