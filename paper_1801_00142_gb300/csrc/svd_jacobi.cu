@@ -37,7 +37,8 @@
 // of FP64 (two FMAs a clock each), run as a cooperative grid with a bounded
 // barrier (on expiry the kernel records a timeout and every CTA leaves).
 // Measured, one FP64 doubling at L = 32, D* = 40, one sweep (62 splits of up
-// to 160 x 160): 1089 ms with Jacobi on C_E, 154 ms with this split.
+// to 160 x 160): 988 ms with Jacobi on C_E, 114 ms with this split (an average
+// split of its bulk takes 0.7 ms: 90 QR steps and some 400 rounds).
 #include <math.h>
 
 #include "common.cuh"
@@ -126,29 +127,55 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-// The rotation that zeroes the Gram entry ga of two columns with squared
-// norms al, be: t = sign(z) / (|z| + sqrt(1 + z^2)), z = (be - al) / (2 ga).
-// FP64 divisions and square roots are long sequences on a pipe of two lanes,
-// so t is computed in FP32 (its error of 1e-7 leaves 1e-7 ga behind, which a
-// later visit removes) and c, s from it to FP64 accuracy (two Newton steps).
-// false: the angle is below FP32's range (nothing to rotate).
-__device__ __forceinline__ bool rotation(double al, double be, double ga, double& t, double& c,
+__device__ __forceinline__ int biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// FP32 value of x 2^(1023 - e0), e0 a biased exponent, by integer operations
+__device__ __forceinline__ float scaled_float(double x, int e0) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ff) - e0 + 127;
+  const unsigned m = ((h & 0xfffffu) << 3) | (l >> 29);
+  const unsigned v = e <= 0 ? 0u : (e >= 255 ? 0x7f800000u : ((unsigned)e << 23) | m);
+  return __uint_as_float((h & 0x80000000u) | v);
+}
+// a normal FP32 value as FP64
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u)),
+                          (int)(u << 29));
+}
+
+// Whether ga^2 > tol2 al be (al, be squared norms, ga their Gram entry):
+// mantissas in FP32, exponents apart.
+__device__ __forceinline__ bool above_tol(double al, double be, double ga, float tol2) {
+  const int eg = biased_exp(ga), ea = biased_exp(al), eb = biased_exp(be);
+  if (eg == 0 || ea == 0 || eb == 0) return false;
+  const float g = scaled_float(ga, eg);
+  const int de = 2 * eg - ea - eb;   // cos^2 = g^2 / (mantissas of al, be) 2^de
+  return de > -140 && g * g * exp2f((float)(de < 100 ? de : 100)) >
+                          tol2 * scaled_float(al, ea) * scaled_float(be, eb);
+}
+
+// The rotation that zeroes the Gram entry ga, as three shears
+//   x -= tau y,  y += s x,  x -= tau y,   tau = tan(theta / 2), s = 2 tau / (1 + tau^2):
+// three FMAs an element where the plain form takes four operations, and no
+// square root.  A warp gets one FP64 instruction through in 64 clocks whatever
+// it is (measured; an ALU instruction takes 5), so the angle, t = tan(theta) =
+// sign(z) / (|z| + sqrt(1 + z^2)), z = (be - al) / (2 ga), comes from FP32 (its
+// error of 1e-7 leaves 1e-7 ga behind, which a later visit removes), the
+// conversions are integer operations, and s follows from tau to FP64 accuracy
+// by one third-order step.  false: the angle is below FP32's range.
+__device__ __forceinline__ bool rotation(double al, double be, double ga, double& t, double& tau,
                                          double& s) {
-  const int e = (__double2hiint(ga) >> 20) & 0x7ff;
-  if (e < 1 || e > 2045) return false;
-  const double sc = __hiloint2double((2046 - e) << 20, 0);   // |ga| sc in [1, 2)
-  const float g = (float)(ga * sc), d = (float)((be - al) * sc);
-  const float z = d / (2.f * g);
-  const float t32 = fabsf(z) > 1e9f ? 0.5f / z
-                                    : copysignf(1.f / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))), z);
-  if (t32 == 0.f) return false;
-  t = (double)t32;
-  const double w = fma(t, t, 1.0);
-  double x = (double)rsqrtf((float)w);
-  x = x * fma(-0.5 * w, x * x, 1.5);
-  x = x * fma(-0.5 * w, x * x, 1.5);
-  c = x;
-  s = x * t;
+  const int eg = biased_exp(ga);
+  const float z = 0.5f * scaled_float(be - al, eg) / scaled_float(ga, eg);
+  const float t32 = fabsf(z) > 1e9f
+                        ? 0.5f / z
+                        : copysignf(1.f / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))), z);
+  if (!(fabsf(t32) > 1e-37f)) return false;
+  const float cf = rsqrtf(fmaf(t32, t32, 1.f)), tf = t32 * cf / (1.f + cf);
+  t = widen(t32);
+  tau = widen(tf);
+  const double w = fma(tau, tau, 1.0), y0 = widen(1.f / fmaf(tf, tf, 1.f)), e = fma(-w, y0, 1.0);
+  s = widen(2.f * tf) * fma(y0, fma(e, e, e), y0);
   return true;
 }
 
@@ -159,7 +186,7 @@ __device__ __forceinline__ int rotate_pair(const SvdArgs& a, int jp, int jq, dou
   double* wp = a.W + (long long)jp * p;
   double* wq = a.W + (long long)jq * p;
   const double al = __ldcg(a.nrm + jp), be = __ldcg(a.nrm + jq);
-  double t, c, s;
+  double t, tau, s;
   if (p <= 32 * REGS) {
     double x[REGS], y[REGS], ga = 0.0;
 #pragma unroll
@@ -172,37 +199,44 @@ __device__ __forceinline__ int rotate_pair(const SvdArgs& a, int jp, int jq, dou
     for (int u = 0; u < REGS; ++u)
       if (32 * u < p) ga = fma(x[u], y[u], ga);
     ga = warp_sum(ga);
-    if (!(ga * ga > a.tol2 * al * be) || !(fabs(ga) > gfloor)) return 0;
-    if (!rotation(al, be, ga, t, c, s)) return 0;
+    if (!above_tol(al, be, ga, (float)a.tol2) || (gfloor > 0.0 && !(fabs(ga) > gfloor))) return 0;
+    if (!rotation(al, be, ga, t, tau, s)) return 0;
 #pragma unroll
     for (int u = 0; u < REGS; ++u) {
       const int e = lane + 32 * u;
-      if (32 * u < p && e < p) {
-        __stcg(wp + e, fma(c, x[u], -(s * y[u])));
-        __stcg(wq + e, fma(s, x[u], c * y[u]));
+      if (32 * u < p) {
+        x[u] = fma(-tau, y[u], x[u]);
+        y[u] = fma(s, x[u], y[u]);
+        x[u] = fma(-tau, y[u], x[u]);
+        if (e < p) {
+          __stcg(wp + e, x[u]);
+          __stcg(wq + e, y[u]);
+        }
       }
     }
     if (lane == 0) {
-      __stcg(a.nrm + jp, fmax(0.0, fma(-t, ga, al)));
-      __stcg(a.nrm + jq, fmax(0.0, fma(t, ga, be)));
+      const double na = fma(-t, ga, al), nb = fma(t, ga, be);
+      __stcg(a.nrm + jp, na > 0.0 ? na : 0.0);
+      __stcg(a.nrm + jq, nb > 0.0 ? nb : 0.0);
     }
-    return 1;
-  }
-  double ga = 0.0;
+  } else {
+    double ga0 = 0.0;
 #pragma unroll 4
-  for (int e = lane; e < p; e += 32) ga = fma(__ldcg(wp + e), __ldcg(wq + e), ga);
-  ga = warp_sum(ga);
-  if (!(ga * ga > a.tol2 * al * be) || !(fabs(ga) > gfloor)) return 0;
-  if (!rotation(al, be, ga, t, c, s)) return 0;
+    for (int e = lane; e < p; e += 32) ga0 = fma(__ldcg(wp + e), __ldcg(wq + e), ga0);
+    const double ga = warp_sum(ga0);
+    if (!above_tol(al, be, ga, (float)a.tol2) || (gfloor > 0.0 && !(fabs(ga) > gfloor))) return 0;
+    if (!rotation(al, be, ga, t, tau, s)) return 0;
 #pragma unroll 4
-  for (int e = lane; e < p; e += 32) {
-    const double x = __ldcg(wp + e), y = __ldcg(wq + e);
-    __stcg(wp + e, fma(c, x, -(s * y)));
-    __stcg(wq + e, fma(s, x, c * y));
-  }
-  if (lane == 0) {
-    __stcg(a.nrm + jp, fmax(0.0, fma(-t, ga, al)));
-    __stcg(a.nrm + jq, fmax(0.0, fma(t, ga, be)));
+    for (int e = lane; e < p; e += 32) {
+      const double y = __ldcg(wq + e), x = fma(-tau, y, __ldcg(wp + e)), yn = fma(s, x, y);
+      __stcg(wq + e, yn);
+      __stcg(wp + e, fma(-tau, yn, x));
+    }
+    if (lane == 0) {
+      const double na = fma(-t, ga, al), nb = fma(t, ga, be);
+      __stcg(a.nrm + jp, na > 0.0 ? na : 0.0);
+      __stcg(a.nrm + jq, nb > 0.0 ? nb : 0.0);
+    }
   }
   return 1;
 }
@@ -230,6 +264,15 @@ __device__ void project(const double* P, long long pi, long long pt, const doubl
     }
     if (i0 + ty < ni && j0 + tx < nj) C[(i0 + ty) * ci + (j0 + tx) * cj] = acc;
   }
+}
+
+constexpr int LGQ = 16;    // lanes of a column in the QR step
+constexpr int REGQ = 16;   // columns up to LGQ * REGQ rows stay in registers there
+
+__device__ __forceinline__ double group_sum(double v) {   // over LGQ lanes
+#pragma unroll
+  for (int o = LGQ / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 template <bool CLUSTER>
@@ -275,102 +318,122 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
     return;
   }
 
-  // ---- 1. pivoted QR (modified Gram-Schmidt), rows of R into W's columns
+  // ---- 1. pivoted QR (modified Gram-Schmidt), rows of R into W's columns;
+  // half a warp per column: an SM gets an FP64 instruction through in 19
+  // clocks and a warp in 64, so the sums over lanes and the scalars count
   int r = 0;
-  double mx0 = 0.0, scale = 1.0, rho_k = -1.0, rem = 0.0;
-  const double nstop = 0.01 * a.rel_tol * a.rel_tol;
+  double scale = 1.0, rem = 0.0;
+  float mx0 = 0.f, rho_k = -1.f, remf = 0.f;   // weights relative to 2^(e0 - 1023) in FP32
+  const int e0 = biased_exp(fro);
+  const float nstop = (float)(0.01 * a.rel_tol * a.rel_tol);
+  const int grp = lane / LGQ, gl = lane % LGQ;
   for (int j = 0; j < a.rmax; ++j) {
     const double* nr = a.nrm + (j & 1) * (long long)a.max_cols;
     double* nw = a.nrm + ((j + 1) & 1) * (long long)a.max_cols;
-    // pivot: the column with the largest norm left (finished ones hold -1);
-    // every warp scans the same values, so all take the same branches
-    double best = -1.0;
+    // pivot: the column with the largest norm left, ties to the lowest column
+    // (finished ones hold -1; positive doubles order like their bits); every
+    // warp scans the same values, so all take the same branches
+    long long best = -1;
     int piv = 0x7fffffff;
-    rem = 0.0;
+    remf = 0.f;
 #pragma unroll 4
     for (int c = lane; c < p; c += 32) {
       const double v = __ldcg(nr + c);
-      if (v > 0.0) rem += v;
-      if (v > best) {
-        best = v;
+      const long long bits = __double_as_longlong(v);
+      if (bits > 0) remf += scaled_float(v, e0);
+      if (bits > best) {
+        best = bits;
         piv = c;
       }
     }
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double v = __shfl_xor_sync(0xffffffffu, best, o);
+      const long long v = __shfl_xor_sync(0xffffffffu, best, o);
       const int c = __shfl_xor_sync(0xffffffffu, piv, o);
+      remf += __shfl_xor_sync(0xffffffffu, remf, o);
       if (v > best || (v == best && c < piv)) {
         best = v;
         piv = c;
       }
     }
-    rem = warp_sum(rem);
-    if (j == 0) {
-      mx0 = best;
+    const double bn = __longlong_as_double(best);
+    if (j == 0 && best > 0) {
+      mx0 = scaled_float(bn, e0);
       // W is scaled by a power of two to norms of at most about 1
-      if (best > 0.0) scale = ldexp(1.0, -(ilogb(best) / 2));
+      scale = ldexp(1.0, -(ilogb(bn) / 2));
     }
-    if (!(best > 0.0) || rem <= nstop * mx0) break;
-    if (j == a.kcap) rho_k = rem;
-    if (rho_k >= 0.0 && j > a.kcap && rem <= 1e-12 * rho_k) break;
-    const double rinv = rsqrt(best);
+    if (best <= 0 || remf <= nstop * mx0) break;
+    if (j == a.kcap) rho_k = remf;
+    if (rho_k >= 0.f && j > a.kcap && remf <= 1e-12f * rho_k) break;
+    // 1 / |pivot|: FP32 for the mantissa (in [1, 4), even exponent), then one
+    // third-order step
+    const int eb = biased_exp(bn), h = (eb - 1023) >> 1;   // bn = m 4^h
+    double rinv;
+    if (eb > 0) {
+      const double m = __hiloint2double(__double2hiint(bn) - (h << 21), __double2loint(bn));
+      const double y0 = widen(rsqrtf(scaled_float(m, 1023)));
+      const double e = fma(-m * y0, y0, 1.0);
+      const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
+      rinv = __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
+    } else {
+      rinv = rsqrt(bn);   // subnormal
+    }
+    const double ws = rinv * scale, binv = rinv * rinv;
     const double* xp = a.A + (long long)piv * q;
     double* wrow = a.W + (long long)j * p;
-    for (int c = gw; c < p; c += TW) {
-      const double nc = __ldcg(nr + c);
-      if (nc < 0.0 || c == piv) {
-        if (lane == 0) {
-          __stcg(wrow + c, c == piv ? best * rinv * scale : 0.0);
-          __stcg(nw + c, -1.0);
-        }
-        continue;
-      }
-      double* xc = a.A + (long long)c * q;
+    double x[REGQ];
+    if (q <= LGQ * REGQ) {
+#pragma unroll
+      for (int u = 0; u < REGQ; ++u) x[u] = gl + LGQ * u < q ? __ldcg(xp + gl + LGQ * u) : 0.0;
+    }
+    for (int c0 = gw * (32 / LGQ); c0 < p; c0 += TW * (32 / LGQ)) {
+      const int c = c0 + grp;
+      const bool in = c < p;
+      const long long nc = in ? __double_as_longlong(__ldcg(nr + c)) : -1;
+      const bool work = nc >= 0 && c != piv;
+      double* xc = a.A + (long long)(in ? c : 0) * q;
       double dot = 0.0, s2 = 0.0;
-      if (q <= 32 * REGS) {
-        double x[REGS], y[REGS];
+      if (q <= LGQ * REGQ) {
+        double y[REGQ];
 #pragma unroll
-        for (int u = 0; u < REGS; ++u) {
-          const int e = lane + 32 * u;
-          x[u] = e < q ? __ldcg(xp + e) : 0.0;
-          y[u] = e < q ? __ldcg(xc + e) : 0.0;
-        }
+        for (int u = 0; u < REGQ; ++u)
+          y[u] = (work && gl + LGQ * u < q) ? __ldcg(xc + gl + LGQ * u) : 0.0;
 #pragma unroll
-        for (int u = 0; u < REGS; ++u)
-          if (32 * u < q) dot = fma(x[u], y[u], dot);
-        dot = warp_sum(dot) * rinv;
-        const double f = dot * rinv;
+        for (int u = 0; u < REGQ; ++u)
+          if (LGQ * u < q) dot = fma(x[u], y[u], dot);
+        dot = group_sum(dot);
+        const double f = dot * binv;
 #pragma unroll
-        for (int u = 0; u < REGS; ++u) {
-          const int e = lane + 32 * u;
-          if (32 * u < q) {
+        for (int u = 0; u < REGQ; ++u)
+          if (LGQ * u < q) {
             y[u] = fma(-f, x[u], y[u]);
             s2 = fma(y[u], y[u], s2);
-            if (e < q) __stcg(xc + e, y[u]);
+            if (work && gl + LGQ * u < q) __stcg(xc + gl + LGQ * u, y[u]);
           }
-        }
       } else {
-#pragma unroll 4
-        for (int e = lane; e < q; e += 32) dot = fma(__ldcg(xp + e), __ldcg(xc + e), dot);
-        dot = warp_sum(dot) * rinv;
-        const double f = dot * rinv;
-#pragma unroll 4
-        for (int e = lane; e < q; e += 32) {
-          const double y = fma(-f, __ldcg(xp + e), __ldcg(xc + e));
-          s2 = fma(y, y, s2);
-          __stcg(xc + e, y);
-        }
+        if (work)
+          for (int e = gl; e < q; e += LGQ) dot = fma(__ldcg(xp + e), __ldcg(xc + e), dot);
+        dot = group_sum(dot);
+        const double f = dot * binv;
+        if (work)
+          for (int e = gl; e < q; e += LGQ) {
+            const double y = fma(-f, __ldcg(xp + e), __ldcg(xc + e));
+            s2 = fma(y, y, s2);
+            __stcg(xc + e, y);
+          }
       }
-      s2 = warp_sum(s2);
-      if (lane == 0) {
-        __stcg(wrow + c, dot * scale);
-        __stcg(nw + c, s2);
+      s2 = group_sum(s2);
+      if (in && gl == 0) {
+        __stcg(wrow + c, c == piv ? bn * ws : (work ? dot * ws : 0.0));
+        __stcg(nw + c, work ? s2 : -1.0);
       }
     }
     r = j + 1;
-    rem = 0.0;   // what is left is known at the next step's scan only
+    remf = 0.f;   // what is left is known at the next step's scan only
     if (!all_sync<CLUSTER>(a)) return;
   }
+  // (a finite fro has e0 below 2047, so the factor is finite)
+  rem = (double)remf * __longlong_as_double((long long)(e0 > 0 ? e0 : 1) << 52);
   // the norms become those of W's columns: every warp has read them
   if (!all_sync<CLUSTER>(a)) return;
 
@@ -416,7 +479,8 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
 #pragma unroll 4
         for (int x = lane; x < p; x += 32) ga = fma(__ldcg(wi + x), __ldcg(wj + x), ga);
         ga = warp_sum(ga);
-        off += ga * ga > a.tol2 * __ldcg(a.nrm + i) * __ldcg(a.nrm + jj) && fabs(ga) > gfloor;
+        off += above_tol(__ldcg(a.nrm + i), __ldcg(a.nrm + jj), ga, (float)a.tol2) &&
+               (!(gfloor > 0.0) || fabs(ga) > gfloor);
       }
       if (lane == 0 && off) atomicAdd(a.cnt + 3 + s % 3, off);
       if (!all_sync<CLUSTER>(a)) return;
@@ -447,9 +511,12 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
     const double s2 = j < r ? __ldcg(a.nrm + j) : 0.0;
     int rk = 0;
     if (j < r) {
+      // non-negative doubles order like their bits
+      const long long b2 = __double_as_longlong(s2);
+#pragma unroll 8
       for (int i = 0; i < r; ++i) {
-        const double x = __ldcg(a.nrm + i);
-        rk += x > s2 || (x == s2 && i < j);
+        const long long x = __double_as_longlong(__ldcg(a.nrm + i));
+        rk += x > b2 || (x == b2 && i < j);
       }
     } else {
       rk = j;
@@ -464,7 +531,8 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const double smx = sqrt(mx);
     int cnt = 0;
-    for (int j = lane; j < r; j += 32) cnt += sqrt(__ldcg(a.nrm + j)) > a.rel_tol * smx;
+    const double thr = a.rel_tol * a.rel_tol * mx;
+    for (int j = lane; j < r; j += 32) cnt += __ldcg(a.nrm + j) > thr;
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     int k = cnt < a.kcap ? cnt : a.kcap;
     if (a.run_if) k = a.kcap < a.rmax ? a.kcap : a.rmax;
