@@ -118,7 +118,8 @@ cudaError_t svd_split_f64(const double* M, int m, int n, int kcap, double rel_to
 // of the orthonormal factor).  It then raises acc->disc_max to its
 // discarded weight (non-negative doubles, compared by bit pattern), counts
 // itself in acc->runs and records a timeout (1) or a sweep limit (2) in
-// acc->status (maximum).  Buffers of acc are device memory.
+// acc->status (maximum).  Buffers of acc are device memory.  cleared: the
+// caller has zeroed buf.counter, buf.kept and buf.stats.
 struct SvdDeviceAcc {
   double* disc_max;
   unsigned long long* runs;
@@ -126,7 +127,8 @@ struct SvdDeviceAcc {
 };
 cudaError_t svd_split_f64_if(const double* M, int m, int n, int kcap, SplitMode mode,
                              double* left, double* right, const SvdBuffers& buf, cudaStream_t st,
-                             const double* run_if, double thresh, const SvdDeviceAcc& acc);
+                             const double* run_if, double thresh, const SvdDeviceAcc& acc,
+                             bool cleared = false);
 
 // ---------------------------------------------------------------- MPO kernels
 cudaError_t mpo_exact_product(const double* A, int la, int ra, const double* B, int lb, int rb,

@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 
 #include "mixed_ops.cuh"
+#include "planes.cuh"
 
 namespace {
 
@@ -13,54 +14,6 @@ inline int grid_for(long long n) {
   if (b > 152 * 32) b = 152 * 32;
   if (b < 1) b = 1;
   return (int)b;
-}
-
-// x = hi + lo with hi the FP32 value of x rounded toward zero and lo what is
-// left, to 24 bits.  FP64 instructions and FP64 <-> FP32 conversions run on a
-// pipe of two lanes per SM, 64 times slower than integer ones, so the parts
-// are cut from the bits; x below 2^-74 or above FP32's range takes the slow
-// conversions (where hi and lo round as the format does).
-__device__ __forceinline__ void f64_parts(double x, float& hi, float& lo) {
-  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
-  const int ef = (int)((h >> 20) & 0x7ff) - 896;   // FP32's biased exponent
-  const unsigned sign = h & 0x80000000u;
-  if (ef >= 53 && ef <= 254) {
-    hi = __uint_as_float(sign | ((unsigned)ef << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
-    const float m = (float)(int)(l & 0x1fffffffu);
-    lo = m * __uint_as_float(sign | ((unsigned)(ef - 52) << 23));
-  } else if (((h << 1) | l) == 0) {
-    hi = lo = 0.f;
-  } else {
-    hi = (float)x;
-    lo = (float)(x - (double)hi);
-  }
-}
-__device__ __forceinline__ void parts(double x, float& hi, float& lo) { f64_parts(x, hi, lo); }
-__device__ __forceinline__ void parts(float x, float& hi, float& lo) {
-  hi = x;
-  lo = 0.f;
-}
-
-// the BF16 planes of x: p0 + p1 + p2 = x to 2^-26
-template <typename S>
-__device__ __forceinline__ void cut(S x, unsigned short* w) {
-  float hi, lo;
-  parts(x, hi, lo);
-  const __nv_bfloat16 p0 = __float2bfloat16_rn(hi);
-  const float r1 = (hi - __bfloat162float(p0)) + lo;
-  const __nv_bfloat16 p1 = __float2bfloat16_rn(r1);
-  const __nv_bfloat16 p2 = __float2bfloat16_rn(r1 - __bfloat162float(p1));
-  w[0] = __bfloat16_as_ushort(p0);
-  w[1] = __bfloat16_as_ushort(p1);
-  w[2] = __bfloat16_as_ushort(p2);
-}
-
-// offset of a view's index with 32-bit divisions (indices are below 2^31)
-__device__ __forceinline__ long long off32(const Idx3& d, unsigned idx) {
-  if (d.n0 == 1 && d.n1 == 1) return (long long)idx * d.s2;
-  const unsigned t = idx / (unsigned)d.n0, i0 = idx - t * (unsigned)d.n0;
-  const unsigned i2 = t / (unsigned)d.n1, i1 = t - i2 * (unsigned)d.n1;
-  return (long long)i2 * d.s2 + (long long)i1 * d.s1 + (long long)i0 * d.s0;
 }
 
 // out[b][r][k] (row stride ld, batch stride obs, plane stride ops) =
@@ -80,7 +33,9 @@ template <typename S>
 __global__ void __launch_bounds__(256)
     to_planes_kernel(const S* __restrict__ src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                      int tiles_r, int tiles_k, long long tiles, __nv_bfloat16* __restrict__ out,
-                     long long ld, long long obs, int planes, long long ops, int kfast, int vec) {
+                     long long ld, long long obs, int planes, long long ops, int kfast, int vec,
+                     const double* __restrict__ run_if, double thresh) {
+  if (run_if && *run_if <= thresh) return;
   __shared__ __align__(16) unsigned short tp[3][TP_R][TP_K + 8];
   const int tid = threadIdx.x;
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -141,7 +96,8 @@ int unit_stride(const Idx3& d) {
 template <typename S>
 cudaError_t launch_to_planes(const S* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                              int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
-                             long long ops, cudaStream_t st) {
+                             long long ops, cudaStream_t st, const double* run_if = nullptr,
+                             double thresh = 0.0) {
   if ((long long)rows * ld * batch <= 0) return cudaSuccess;
   const int tiles_r = (rows + TP_R - 1) / TP_R, tiles_k = (int)((ld + TP_K - 1) / TP_K);
   const long long tiles = (long long)tiles_r * tiles_k * batch;
@@ -150,7 +106,8 @@ cudaError_t launch_to_planes(const S* src, Idx3 rv, Idx3 kv, long long sbs, int 
   const long long grid = tiles < 152 * 16 ? tiles : 152 * 16;
   note_launch();
   to_planes_kernel<S><<<(unsigned)grid, 256, 0, st>>>(src, rv, kv, sbs, rows, K, tiles_r, tiles_k,
-                                                      tiles, out, ld, obs, planes, ops, kfast, vec);
+                                                      tiles, out, ld, obs, planes, ops, kfast, vec, run_if,
+                                                      thresh);
   return cudaGetLastError();
 }
 
@@ -272,6 +229,14 @@ cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int ro
   return launch_to_planes<double>(src, rv, kv, sbs, rows, K, batch, out, ld, obs, planes, ops, st);
 }
 
+cudaError_t to_planes_if(const double* src, Idx3 rv, Idx3 kv, int rows, int K, __nv_bfloat16* out,
+                         long long ld, int planes, long long ops, const double* run_if,
+                         double thresh, cudaStream_t st) {
+  if (!run_if) return cudaErrorInvalidValue;
+  return launch_to_planes<double>(src, rv, kv, 0, rows, K, 1, out, ld, 0, planes, ops, st, run_if,
+                                  thresh);
+}
+
 cudaError_t to_planes_f32(const float* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                           int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                           long long ops, cudaStream_t st) {
@@ -290,8 +255,6 @@ cudaError_t reduce_partials_planes(const float* part, int splits, int m, int n, 
                                    __nv_bfloat16* prm, long long ldn, __nv_bfloat16* ptr,
                                    long long ldm, long long ps, double* ss, cudaStream_t st) {
   if (m <= 0 || n <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(double), st);
-  if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((n + 31) / 32), (unsigned)((m + 31) / 32));
   note_launch();
   reduce_partials_planes_kernel<<<grid, 256, 0, st>>>(part, splits, m, n, out, prm, ldn, ptr, ldm,

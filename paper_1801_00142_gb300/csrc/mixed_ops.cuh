@@ -9,6 +9,10 @@
 cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                       int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                       long long ops, cudaStream_t st);
+// to_planes of one matrix, run only if *run_if > thresh or is not finite.
+cudaError_t to_planes_if(const double* src, Idx3 rv, Idx3 kv, int rows, int K, __nv_bfloat16* out,
+                         long long ld, int planes, long long ops, const double* run_if,
+                         double thresh, cudaStream_t st);
 cudaError_t to_planes_f32(const float* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                           int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                           long long ops, cudaStream_t st);
@@ -17,7 +21,8 @@ cudaError_t reduce_partials(const float* part, int splits, long long n, double* 
                             cudaStream_t st);
 // C = sum of the split-K partials (m x n): FP64 into out, the three BF16
 // planes (plane stride ps) row-major into prm [m][ldn] and transposed into
-// ptr [n][ldm] (zero padding), and ||C||_F^2 into *ss (device scalar).
+// ptr [n][ldm] (zero padding), and ||C||_F^2 added to *ss (device scalar,
+// which the caller has cleared).
 cudaError_t reduce_partials_planes(const float* part, int splits, int m, int n, double* out,
                                    __nv_bfloat16* prm, long long ldn, __nv_bfloat16* ptr,
                                    long long ldm, long long ps, double* ss, cudaStream_t st);

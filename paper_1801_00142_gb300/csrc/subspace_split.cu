@@ -39,6 +39,7 @@
 
 #include "common.cuh"
 #include "mixed_ops.cuh"
+#include "planes.cuh"
 #include "subspace_split.cuh"
 #include "tc_gemm.cuh"
 
@@ -57,7 +58,7 @@ __device__ inline float hash_uniform(unsigned long long x) {
   x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
   x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
   x ^= x >> 31;
-  return (float)((double)(x >> 11) * (1.0 / 9007199254740992.0) * 2.0 - 1.0);
+  return (float)(unsigned)(x >> 40) * (1.f / 8388608.f) - 1.f;   // 24 bits, no FP64
 }
 
 // Q[r][j] (rows x k) = src(j, r) for j < kold (src FP64 with strides), else
@@ -940,20 +941,33 @@ __global__ void __launch_bounds__(CQ_NT, 1)
   if (tid == 0 && ndefl) atomicAdd(flag + 4, ndefl);
 }
 
+// BF16 planes of U and U^T (3 planes each; both null: not wanted).
+struct SolvePlanes {
+  __nv_bfloat16* rm;   // [plane][rows][ldk], plane stride ps_rm
+  long long ldk, ps_rm;
+  __nv_bfloat16* tr;   // [plane][k][ldr], plane stride ps_tr
+  long long ldr, ps_tr;
+};
+
 // U[r] = (Y[r] o d) L^{-T} for every row r (one warp per row; rows ldy / ldu
 // apart, so a column block of a wider matrix works in place): with u L^T = z,
 // u_j = (z_j - sum_{i<j} u_i L_ji) / L_jj, in blocks of 32 columns (earlier
 // blocks first, then a sequential solve inside the block).  Does nothing if
 // *flag is set (the fast path broke down) or, with run_if set, if *run_if is
 // 0.  U may be Y itself (ldu = ldy): each row is read by the lanes that
-// write it, column j before U[r][j].
+// write it, column j before U[r][j].  With planes, U's and U^T's BF16 planes
+// are written too, the operands of the next two products (the eight rows of
+// a CTA are one 16-byte store per column of U^T).
 __global__ void __launch_bounds__(CQ_SOLVE_NT)
     cholqr_solve(const float* Y, long long ldy, int rows, int k,
                  const float* __restrict__ Lp, const float* __restrict__ dv,
                  const float* __restrict__ linv, const int* __restrict__ flag,
-                 const int* __restrict__ run_if, float* U, long long ldu) {
+                 const int* __restrict__ run_if, float* U, long long ldu, SolvePlanes pl) {
   if (*flag || (run_if && *run_if == 0)) return;
   extern __shared__ __align__(16) float Ls[];
+  constexpr int WPB = CQ_SOLVE_NT / 32;
+  static_assert(WPB == 8, "eight rows a CTA: one 16-byte store per column and plane");
+  __shared__ __align__(16) unsigned short tp[3][MAX_K][WPB];
   const int np = k * (k + 1) / 2;
   // the packed factor (16-byte aligned in global memory), 16 bytes per load
   const int n4 = np / 4;
@@ -962,16 +976,17 @@ __global__ void __launch_bounds__(CQ_SOLVE_NT)
     reinterpret_cast<float4*>(Ls)[e] = reinterpret_cast<const float4*>(Lp)[e];
   for (int e = 4 * n4 + threadIdx.x; e < np; e += CQ_SOLVE_NT) Ls[e] = Lp[e];
   __syncthreads();
-  const int lane = threadIdx.x % 32;
-  const int WPB = CQ_SOLVE_NT / 32;
-  for (int r = blockIdx.x * WPB + threadIdx.x / 32; r < rows; r += gridDim.x * WPB) {
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  for (int r0 = blockIdx.x * WPB; r0 < rows; r0 += gridDim.x * WPB) {
+    const int r = r0 + warp;
+    const bool in = r < rows;
     float x[MAX_K / 32];
 #pragma unroll
     for (int qb = 0; qb < MAX_K / 32; ++qb) {
       x[qb] = 0.f;
       if (qb * 32 < k) {
         const int j = qb * 32 + lane;
-        float s = (j < k) ? Y[(long long)r * ldy + j] * dv[j] : 0.f;
+        float s = (in && j < k) ? Y[(long long)r * ldy + j] * dv[j] : 0.f;
         // earlier blocks
 #pragma unroll
         for (int q = 0; q < MAX_K / 32; ++q) {
@@ -996,8 +1011,28 @@ __global__ void __launch_bounds__(CQ_SOLVE_NT)
           }
         }
         x[qb] = xj;
-        if (j < k) U[(long long)r * ldu + j] = xj;
+        if (in && j < k) U[(long long)r * ldu + j] = xj;
+        if (pl.rm && j < pl.ldk) {
+          unsigned short w[3] = {0, 0, 0};
+          if (j < k) cut(xj, w);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            if (in) pl.rm[q * pl.ps_rm + (long long)r * pl.ldk + j] = __ushort_as_bfloat16(w[q]);
+            tp[q][j][warp] = w[q];
+          }
+        }
       }
+    }
+    if (pl.rm) {
+      __syncthreads();
+      // rows past the last one were zero, as the padding of U^T has to be
+      if (r0 < pl.ldr)
+        for (int e = threadIdx.x; e < 3 * k; e += CQ_SOLVE_NT) {
+          const int q = e / k, j = e - q * k;
+          *reinterpret_cast<uint4*>(pl.tr + q * pl.ps_tr + (long long)j * pl.ldr + r0) =
+              *reinterpret_cast<const uint4*>(tp[q][j]);
+        }
+      __syncthreads();
     }
   }
 }
@@ -1083,7 +1118,7 @@ cudaError_t cholqr2_block(float* Yb, long long ldy, int rows, int w, float* tmp,
     RET(cudaGetLastError());
     note_launch();
     cholqr_solve<<<grid, CQ_SOLVE_NT, ssm, st>>>(src, lds, rows, w, b.chol_L, b.chol_d, b.chol_li,
-                                                 b.chol_flag, nullptr, dst, ldd);
+                                                 b.chol_flag, nullptr, dst, ldd, SolvePlanes{});
     RET(cudaGetLastError());
     src = tmp;
     lds = w;
@@ -1110,40 +1145,62 @@ __global__ void subtract_block_kernel(float* __restrict__ Yb, long long ldy,
 // of U1 is G2 = I + E with E small; its Cholesky factor is L = I + Phi(E) +
 // O(E^2), Phi(E) the strictly lower part of E plus half its diagonal, so
 // U2 = U1 L^{-T} = U1 (I - Phi(E)^T) + O(E^2) and U2^T U2 = I + O(E^2).
-// Writes B = I - Phi(E) (k x k row-major: U2 = U1 B^T is one tensor-core
-// product); dead columns (G2_jj < 1/2, zero columns of U1) keep B's row e_j
+// Writes B = I - Phi(E) (k x k: U2 = U1 B^T is one tensor-core product);
+// dead columns (G2_jj < 1/2, zero columns of U1) keep B's row e_j
 // and get zeros elsewhere.  If a live |E_ij| exceeds emax (or is not
 // finite), sets *need_full: the full second pass runs instead (and counts
 // itself in need_full[1]).
-__global__ void cholqr_linear_kernel(const float* __restrict__ G, int k, float emax,
-                                     float* __restrict__ B, int* need_full) {
-  bool big = false;
-  const long long total = (long long)k * k;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int n = (int)(e / k), c = (int)(e % k);
-    const float gn = G[(long long)n * k + n], gc = G[(long long)c * k + c];
-    const bool ln = gn >= 0.5f, lc = gc >= 0.5f;
+// G comes as the partials of its split contraction: summed here, with the
+// sum written to G for the full second pass; B as its BF16 planes.
+__global__ void __launch_bounds__(256)
+    cholqr_linear_kernel(const float* __restrict__ part, int splits, int k, float emax,
+                         float* __restrict__ G, __nv_bfloat16* __restrict__ B, long long ldb,
+                         long long psb, int* need_full) {
+  __shared__ float dn[32], dc[32];
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int n0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const long long kk = (long long)k * k;
+  auto sum = [&](long long e) {
     float v = 0.f;
-    if (!ln) {
-      v = (n == c) ? 1.f : 0.f;
-    } else if (lc) {
-      const float E = (n == c) ? gn - 1.f : G[e];
-      if (!(fabsf(E) <= emax)) big = true;
-      v = (n == c) ? 1.f - 0.5f * E : (n > c ? -E : 0.f);
+#pragma unroll 8
+    for (int s = 0; s < splits; ++s) v += part[s * kk + e];
+    return v;
+  };
+  // the diagonal entries of the tile's rows and columns
+  if (ty < 2) {
+    const int i = (ty ? c0 : n0) + tx;
+    (ty ? dc : dn)[tx] = i < k ? sum((long long)i * k + i) : 0.f;
+  }
+  float g[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int n = n0 + ty + 8 * u, c = c0 + tx;
+    g[u] = (n < k && c < k) ? sum((long long)n * k + c) : 0.f;
+  }
+  __syncthreads();
+  bool big = false;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int n = n0 + ty + 8 * u, c = c0 + tx;
+    if (n >= k || c >= ldb) continue;
+    const float gn = dn[ty + 8 * u], gc = dc[tx];
+    float v = 0.f;
+    if (c < k) {
+      if (!(gn >= 0.5f)) {
+        v = (n == c) ? 1.f : 0.f;
+      } else if (gc >= 0.5f) {
+        const float E = (n == c) ? gn - 1.f : g[u];
+        if (!(fabsf(E) <= emax)) big = true;
+        v = (n == c) ? 1.f - 0.5f * E : (n > c ? -E : 0.f);
+      }
+      G[(long long)n * k + c] = g[u];
     }
-    B[e] = v;
+    unsigned short w[3];
+    cut(v, w);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) B[q * psb + (long long)n * ldb + c] = __ushort_as_bfloat16(w[q]);
   }
   if (__syncthreads_or(big) && threadIdx.x == 0) atomicExch(need_full, 1);
-}
-
-// dst[r][c] = src[r][c] (rows x k, contiguous) if *flag != 0
-__global__ void copy_if_flag_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                    long long n, const int* __restrict__ flag) {
-  if (*flag == 0) return;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    dst[e] = src[e];
 }
 
 // Largest |E_ij| of the first-order second pass; above it the full second
@@ -1153,75 +1210,18 @@ __global__ void copy_if_flag_kernel(const float* __restrict__ src, float* __rest
 // checked basis was measured not to change the free energy.
 constexpr float CQ_LINEAR_EMAX = 1e-3f;
 
-// An orthonormal basis of the columns of Y (rows x k, FP32), written to
-// *U (b.Q or Y itself); Y and b.Q are overwritten.  Up to one column block
-// (k <= b.orth_block): scaled CholeskyQR2 with its second pass to first order
-// (Y -> U1 in place, then U2 = U1 B^T into b.Q, see cholqr_linear_kernel);
-// the full second pass runs instead when U1 is too far from orthonormal, and
-// the block Gram-Schmidt kernels when a pass breaks down (all chosen on the
-// device by flags; see cholqr_factor).  Wider: block classical Gram-Schmidt
-// over column blocks, each projected twice against the blocks before it on
-// the tensor cores (S = Q^T Y_b, Y_b -= Q S) and then orthonormalised by
-// scaled CholeskyQR2, result in Y; a breakdown leaves Y unorthonormal, which
-// the caller's orthonormality check turns into the exact split.
-cudaError_t orthonormalise(float* Y, int rows, int k, const SubspaceBuffers& b, cudaStream_t st,
-                           float** U) {
+// An orthonormal basis of the columns of Y (rows x k, FP32) for k wider than
+// one column block, in place: block classical Gram-Schmidt over column blocks,
+// each projected twice against the blocks before it on the tensor cores (S =
+// Q^T Y_b, Y_b -= Q S) and then orthonormalised by scaled CholeskyQR2; a
+// breakdown leaves Y unorthonormal, which the caller's orthonormality check
+// turns into the exact split.  b.Q is overwritten.
+cudaError_t orthonormalise_blocks(float* Y, int rows, int k, const SubspaceBuffers& b,
+                                  cudaStream_t st) {
   if (k > SUBSPACE_MAX_K) return cudaErrorInvalidValue;
   RET(cholqr_setup());
-  // chol_flag: [0] breakdown, [1] breakdowns counted by the block Gram-Schmidt
-  // kernels, [2] full second pass needed, [3] full second passes counted,
-  // [4] columns dropped as numerically dependent by the first pass
-  RET(cudaMemsetAsync(b.chol_flag, 0, sizeof(int), st));
-  RET(cudaMemsetAsync(b.chol_flag + 2, 0, sizeof(int), st));
   const int B = b.orth_block;
   if (B < 32 || B > MAX_K || B % 32) return cudaErrorInvalidValue;
-  if (k <= B) {
-    const size_t fsm = cholqr_factor_smem(k), ssm = (size_t)k * (k + 1) / 2 * 4;
-    const int wpb = CQ_SOLVE_NT / 32;
-    const int grid = (rows + wpb - 1) / wpb < 152 ? (rows + wpb - 1) / wpb : 152;
-    float* G = b.out;                          // k x k Grams
-    float* Bm = b.out + (size_t)k * k;         // k x k first-order factor
-    int* need_full = b.chol_flag + 2;
-    // pass 1: G = Y^T Y, scaled Cholesky, Y <- U1 in place (skipped on breakdown)
-    RET(tc_product(f32_view(Y, idx_plain(1), idx_plain(k)), f32_view(Y, idx_plain(1), idx_plain(k)),
-                   k, k, rows, G, k, b, st));
-    note_launch();
-    cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 1e-6f, 1, b.chol_L, b.chol_d, b.chol_li,
-                                         b.chol_flag, nullptr);
-    RET(cudaGetLastError());
-    note_launch();
-    cholqr_solve<<<grid, CQ_SOLVE_NT, ssm, st>>>(Y, k, rows, k, b.chol_L, b.chol_d, b.chol_li,
-                                                 b.chol_flag, nullptr, Y, k);
-    RET(cudaGetLastError());
-    // pass 2 to first order: G = U1^T U1 = I + E, b.Q <- U1 (I - Phi(E)^T)
-    RET(tc_product(f32_view(Y, idx_plain(1), idx_plain(k)), f32_view(Y, idx_plain(1), idx_plain(k)),
-                   k, k, rows, G, k, b, st));
-    note_launch();
-    cholqr_linear_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(G, k, CQ_LINEAR_EMAX, Bm,
-                                                                     need_full);
-    RET(cudaGetLastError());
-    RET(tc_product(f32_view(Y, idx_plain(k), idx_plain(1)), f32_view(Bm, idx_plain(k), idx_plain(1)),
-                   rows, k, k, b.Q, k, b, st));
-    // the full second pass, only if E was too large: U1 -> b.Q
-    note_launch();
-    cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 0.25f, 0, b.chol_L, b.chol_d, b.chol_li,
-                                         b.chol_flag, need_full);
-    RET(cudaGetLastError());
-    note_launch();
-    cholqr_solve<<<grid, CQ_SOLVE_NT, ssm, st>>>(Y, k, rows, k, b.chol_L, b.chol_d, b.chol_li,
-                                                 b.chol_flag, need_full, b.Q, k);
-    RET(cudaGetLastError());
-    // a breakdown in either pass: block Gram-Schmidt on Y (the input, or U1
-    // after a breakdown of the second pass), copied to b.Q
-    RET(block_cgs(Y, rows, k, b, st, b.chol_flag));
-    note_launch();
-    copy_if_flag_kernel<<<grid_for((long long)rows * k), 256, 0, st>>>(Y, b.Q, (long long)rows * k,
-                                                                       b.chol_flag);
-    RET(cudaGetLastError());
-    *U = b.Q;
-    return cudaSuccess;
-  }
-  *U = Y;
   for (int j0 = 0; j0 < k; j0 += B) {
     const int w = k - j0 < B ? k - j0 : B;
     float* Yb = Y + j0;
@@ -1242,6 +1242,390 @@ cudaError_t orthonormalise(float* Y, int rows, int k, const SubspaceBuffers& b, 
   return cudaSuccess;
 }
 
+// ---------------------------------------------------------------------------
+// The truncation up to one column block (k <= b.orth_block), a chain of
+// kernels each bound by its launch and latency at the bonds met here: every
+// tensor-core product leaves its split-K partials, and the kernel after it
+// sums them and writes the next product's operand planes, so that no pass
+// only sums, converts, copies or clears.  U_hat is the basis kept as planes of
+// its transpose (U^T left-to-right, V^T right-to-left) behind C_E's planes, so
+// that one product gives both the centre and the Gram of the check.
+
+// warm start as planes: out[j][r] = src(j, r) = S[j * sj + r * sr] for j <
+// kold, else pseudo-random (k rows of ld columns).  Clears the scalars of the
+// update (zero_words words at zero, and the two flags).
+__global__ void __launch_bounds__(256)
+    warm_planes_kernel(const double* __restrict__ S, long long sj, long long sr, int kold, int rows,
+                       int k, unsigned long long seed0,
+                       const unsigned long long* __restrict__ base, __nv_bfloat16* __restrict__ out,
+                       long long ld, long long ps, int* zero, int zero_words, int* flags) {
+  __shared__ __align__(16) unsigned short tp[3][32][72];
+  const int tid = threadIdx.x;
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    if (tid < zero_words) zero[tid] = 0;
+    if (tid == 64) flags[0] = 0;
+    if (tid == 65) flags[2] = 0;
+  }
+  const unsigned long long seed = seed0 ^ (*base * 0x9E3779B97F4A7C15ull);
+  const int j0 = blockIdx.y * 32, r0 = blockIdx.x * 64;
+  const bool rfast = sr == 1;
+  double x[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int j = j0 + (rfast ? tid / 64 + 4 * u : tid % 32);
+    const int r = r0 + (rfast ? tid % 64 : tid / 32 + 8 * u);
+    x[u] = (j < kold && r < rows) ? S[j * sj + r * sr] : 0.0;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int y = rfast ? tid / 64 + 4 * u : tid % 32, z = rfast ? tid % 64 : tid / 32 + 8 * u;
+    const int j = j0 + y, r = r0 + z;
+    unsigned short w[3];
+    if (j >= kold && r < rows)
+      cut(hash_uniform(seed * 0x100000001B3ull + (unsigned long long)r * k + j), w);
+    else
+      cut(x[u], w);
+    tp[0][y][z] = w[0];
+    tp[1][y][z] = w[1];
+    tp[2][y][z] = w[2];
+  }
+  __syncthreads();
+  const int y = tid / 8, z = tid % 8 * 8, j = j0 + y, r = r0 + z;
+  if (j < k && r < ld)
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      *reinterpret_cast<uint4*>(out + q * ps + (long long)j * ld + r) =
+          *reinterpret_cast<const uint4*>(&tp[q][y][z]);
+}
+
+// The source of one basis factor (rows x k, row-major FP32): the sum of a
+// product's partials, or a finished array chosen on the device.
+struct BasisSrc {
+  const float* part;
+  int splits;
+  const float* alt1;   // taken instead if *flag1 != 0
+  const int* flag1;
+  const float* alt2;   // taken instead if *flag2 != 0 (and not alt1)
+  const int* flag2;
+};
+
+// F = source (+ noise eta R with eta = 1e-5 rms(C_E)); written as FP32 (f32,
+// may be null), FP64 row-major (f64) or transposed (f64t), and as planes of
+// F^T [plane][k][ldr] (zero padding).  Tiles of 64 rows x 32 columns.
+__global__ void __launch_bounds__(256)
+    basis_kernel(BasisSrc src, int rows, int k, const double* __restrict__ tot, double inv_mn,
+                 unsigned long long seed0, const unsigned long long* __restrict__ base, float* f32,
+                 double* f64, double* f64t, __nv_bfloat16* __restrict__ out, long long ldr,
+                 long long ps) {
+  __shared__ float v[32][65];   // [column][row]
+  const int tid = threadIdx.x, tx = tid % 32, ty = tid / 32;
+  const int r0 = blockIdx.x * 64, j0 = blockIdx.y * 32;
+  const float* alt = nullptr;
+  if (src.flag1 && *src.flag1) alt = src.alt1;
+  else if (src.flag2 && *src.flag2) alt = src.alt2;
+  const long long n = (long long)rows * k;
+  float a[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int r = r0 + ty + 8 * u, j = j0 + tx;
+    a[u] = 0.f;
+    if (alt && r < rows && j < k) a[u] = alt[(long long)r * k + j];
+  }
+  if (!alt) {
+#pragma unroll 2
+    for (int s = 0; s < src.splits; ++s)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int r = r0 + ty + 8 * u, j = j0 + tx;
+        if (r < rows && j < k) a[u] += src.part[s * n + (long long)r * k + j];
+      }
+  }
+  if (tot) {
+    const unsigned long long seed = seed0 ^ (*base * 0x9E3779B97F4A7C15ull);
+    const float eta = (float)(1e-5 * sqrt(*tot * inv_mn));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const long long e = (long long)(r0 + ty + 8 * u) * k + j0 + tx;
+      a[u] += eta * hash_uniform(seed ^ (0xD1B54A32D192ED03ull * (unsigned long long)(e + 1)));
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int r = r0 + ty + 8 * u, j = j0 + tx;
+    const bool in = r < rows && j < k;
+    v[tx][ty + 8 * u] = in ? a[u] : 0.f;
+    if (in && f32) f32[(long long)r * k + j] = a[u];
+    if (in && f64) f64[(long long)r * k + j] = (double)a[u];
+  }
+  __syncthreads();
+  {
+    const int y = tid / 8, z = tid % 8 * 8, j = j0 + y, r = r0 + z;
+    if (j < k && r < ldr) {
+      __align__(16) unsigned short w[3][8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        unsigned short c[3];
+        cut(v[y][z + u], c);
+        w[0][u] = c[0];
+        w[1][u] = c[1];
+        w[2][u] = c[2];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        *reinterpret_cast<uint4*>(out + q * ps + (long long)j * ldr + r) =
+            *reinterpret_cast<const uint4*>(w[q]);
+    }
+  }
+  if (f64t)
+    for (int e = tid; e < 32 * 64; e += 256) {
+      const int j = j0 + e / 64, r = r0 + e % 64;
+      if (j < k && r < rows) f64t[(long long)j * rows + r] = (double)v[e / 64][e % 64];
+    }
+}
+
+// The last product: its partials (R x Cc) hold the centre and, in the columns
+// from c_gram on (left-to-right) or the rows from r_gram on, the Gram of the
+// kept basis.  Writes the centre in FP64 (row stride ldo), adds its sum of
+// squares, raises the orthonormality defect over the live columns; the last
+// CTA to finish sets the defect to +inf when no column is live, raises the
+// discarded weight of an accepted split into *disc_max (may be null) and
+// clears ||C_E||^2 for the next update.
+struct CentreOut {
+  double* out;
+  int ldo, r_gram, c_gram, k;
+  double* dscal;   // [1] sum of squares, [2] defect
+  int* live;       // [0] a live column seen, [1] CTAs finished
+  double* ce_ss;
+  double thresh;
+  double* disc_max;
+};
+__global__ void __launch_bounds__(256)
+    centre_kernel(const float* __restrict__ part, int splits, int R, int Cc, CentreOut o) {
+  __shared__ float dr[32], dc[32];
+  __shared__ double red[8];
+  __shared__ float redf[8];
+  __shared__ int last;
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const long long n = (long long)R * Cc;
+  auto sum = [&](long long e) {
+    float v = 0.f;
+#pragma unroll 8
+    for (int s = 0; s < splits; ++s) v += part[s * n + e];
+    return v;
+  };
+  const bool grams = r0 + 31 >= o.r_gram || c0 + 31 >= o.c_gram;   // some Gram entry in this tile
+  if (grams && ty < 2) {
+    // Gram index of the tile's rows (ty = 0) and columns (ty = 1), and the
+    // diagonal entry there
+    const int i = ty == 0 ? r0 + tx - (o.r_gram < R ? o.r_gram : 0)
+                          : c0 + tx - (o.c_gram < Cc ? o.c_gram : 0);
+    float d = 0.f;
+    if (i >= 0 && i < o.k)
+      d = sum((long long)(i + (o.r_gram < R ? o.r_gram : 0)) * Cc + i +
+              (o.c_gram < Cc ? o.c_gram : 0));
+    (ty ? dc : dr)[tx] = d;
+  }
+  if (grams) __syncthreads();
+  double acc = 0.0;
+  float mx = 0.f;
+  int live = 0;
+  float v4[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = r0 + ty + 8 * u, c = c0 + tx;
+    v4[u] = (r < R && c < Cc) ? sum((long long)r * Cc + c) : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = r0 + ty + 8 * u, c = c0 + tx;
+    if (r >= R || c >= Cc) continue;
+    const float v = v4[u];
+    if (r < o.r_gram && c < o.c_gram) {
+      const double d = (double)v;
+      o.out[(long long)r * o.ldo + c] = d;
+      acc = fma(d, d, acc);
+    } else {
+      const int i = r - (o.r_gram < R ? o.r_gram : 0), j = c - (o.c_gram < Cc ? o.c_gram : 0);
+      const float gi = dr[ty + 8 * u], gj = dc[tx];
+      if (i == j && gi >= 0.5f) live = 1;
+      if (!(gi < 0.5f || gj < 0.5f)) {
+        const float d = fabsf(v - (i == j ? 1.f : 0.f));
+        mx = fmaxf(mx, d != d ? 1e30f : d);
+      }
+    }
+  }
+  for (int s = 16; s > 0; s >>= 1) {
+    acc += __shfl_xor_sync(0xffffffffu, acc, s);
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+  }
+  if (tx == 0) {
+    red[ty] = acc;
+    redf[ty] = mx;
+  }
+  const int any_live = __syncthreads_or(live);
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    float m = 0.f;
+    for (int i = 0; i < 8; ++i) {
+      t += red[i];
+      m = fmaxf(m, redf[i]);
+    }
+    if (t != 0.0) atomicAdd(o.dscal + 1, t);
+    // non-negative doubles order like their bit patterns
+    if (m > 0.f)
+      atomicMax(reinterpret_cast<unsigned long long*>(o.dscal + 2),
+                (unsigned long long)__double_as_longlong((double)m));
+    if (any_live) atomicOr(o.live, 1);
+    __threadfence();
+    last = atomicAdd(o.live + 1, 1) == (int)(gridDim.x * gridDim.y) - 1;
+  }
+  __syncthreads();
+  if (last && threadIdx.x == 0) {
+    __threadfence();
+    const double tot = __ldcg(o.ce_ss), kept = __ldcg(o.dscal + 1);
+    double defect = __ldcg(o.dscal + 2);
+    if (__ldcg(o.live) == 0) {
+      defect = INFINITY;
+      o.dscal[2] = defect;
+    }
+    const double disc = tot > 0.0 ? fmax(0.0, 1.0 - kept / tot) : 0.0;
+    if (o.disc_max && defect <= o.thresh)
+      atomicMax(reinterpret_cast<unsigned long long*>(o.disc_max),
+                (unsigned long long)__double_as_longlong(disc));
+    *o.ce_ss = 0.0;
+  }
+}
+
+// A B^T on the tensor cores (3 planes, 6 products) as split-K partials in
+// b.part; *splits: their number.  Products with few output tiles split K so
+// that about one wave of CTAs runs.
+cudaError_t tc_partials(const TcOperand& A, const TcOperand& B, int M, int N, int K, int* splits,
+                        const SubspaceBuffers& b, cudaStream_t st) {
+  const int kb = (K + 63) / 64, tiles = ((M + 127) / 128) * ((N + 127) / 128);
+  int sk = 1;
+  if (tiles < 76) {
+    sk = 152 / tiles;
+    sk = sk < kb ? sk : kb;
+    sk = sk < 32 ? sk : 32;
+    const int per = (kb + sk - 1) / sk;
+    sk = (kb + per - 1) / per;
+    while (sk > 1 && (size_t)sk * M * N > b.part_floats) --sk;
+  }
+  if ((size_t)sk * M * N > b.part_floats) return cudaErrorInvalidValue;
+  TcOutput o;
+  memset(&o, 0, sizeof o);
+  o.alpha = 1.0;
+  o.mode = TC_OUT_PARTIAL;
+  o.f32 = b.part;
+  *splits = sk;
+  return tc_gemm(A, B, M, N, K, 1, 6, sk, o, b.err, st);
+}
+
+TcOperand plane_op(const __nv_bfloat16* p, int rows, int k, long long ld, long long ps) {
+  return TcOperand{p, 3, rows, k, ld, 0, ps, 1};
+}
+
+cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm, int kold,
+                         double* left, double* right, unsigned long long seed,
+                         const SubspaceBuffers& b, cudaStream_t st, double* disc_max,
+                         double thresh) {
+  RET(cholqr_setup());
+  // the basis has `rows` rows on the side of the isometry, the other side is
+  // `other`; ce: C_E with that side as rows, behind it the basis' transpose
+  const int rows = dir_right ? m : n, other = dir_right ? n : m;
+  const long long ldr = tc_ld(rows), ldo = tc_ld(other), ldk = tc_ld(k);
+  const __nv_bfloat16* ce = dir_right ? b.ce_rm : b.ce_tr;      // rows x other
+  __nv_bfloat16* cet = dir_right ? b.ce_tr : b.ce_rm;           // other x rows
+  __nv_bfloat16* hat = cet + (long long)other * ldr;            // k x rows: the basis, transposed
+  if ((long long)(other + k) * ldr > b.ce_ps || (long long)rows * ldk > b.psa ||
+      (long long)k * ldr > b.psb || (long long)k * ldo > b.psb || (long long)k * ldk > b.psb)
+    return cudaErrorInvalidValue;
+  const size_t fsm = cholqr_factor_smem(k), ssm = (size_t)k * (k + 1) / 2 * 4;
+  const int wpb = CQ_SOLVE_NT / 32;
+  const int sgrid = (rows + wpb - 1) / wpb < 152 ? (rows + wpb - 1) / wpb : 152;
+  const dim3 bgrid((unsigned)((ldr + 63) / 64), (unsigned)((k + 31) / 32));
+  float* G = b.out;
+  int* need_full = b.chol_flag + 2;
+  int sp = 1;
+  // warm start Q^T (k x other): the current C_{i+1} rows or C_i columns
+  note_launch();
+  warm_planes_kernel<<<dim3((unsigned)((ldo + 63) / 64), (unsigned)((k + 31) / 32)), 256, 0, st>>>(
+      warm, dir_right ? n : 1, dir_right ? 1 : kold, kold, other, k, seed, b.seed_base, b.pb, ldo,
+      b.psb, b.zero, b.zero_words, b.chol_flag);
+  RET(cudaGetLastError());
+  // Y = C_E Q (rows x k) + noise, and the planes of Y^T
+  RET(tc_partials(plane_op(ce, rows, other, ldo, b.ce_ps), plane_op(b.pb, k, other, ldo, b.psb), rows,
+                  k, other, &sp, b, st));
+  note_launch();
+  basis_kernel<<<bgrid, 256, 0, st>>>(BasisSrc{b.part, sp, nullptr, nullptr, nullptr, nullptr}, rows,
+                                      k, b.ce_ss, 1.0 / ((double)m * n), seed + 7, b.seed_base, b.Y,
+                                      nullptr, nullptr, hat, ldr, b.ce_ps);
+  RET(cudaGetLastError());
+  // pass 1: G = Y^T Y, scaled Cholesky, Y <- U1 in place (skipped on breakdown)
+  const TcOperand H = plane_op(hat, k, rows, ldr, b.ce_ps);
+  RET(tc_partials(H, H, k, k, rows, &sp, b, st));
+  note_launch();
+  sum_partials_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(b.part, sp, k, k, G, k);
+  note_launch();
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 1e-6f, 1, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+                                       nullptr);
+  RET(cudaGetLastError());
+  note_launch();
+  cholqr_solve<<<sgrid, CQ_SOLVE_NT, ssm, st>>>(b.Y, k, rows, k, b.chol_L, b.chol_d, b.chol_li,
+                                                b.chol_flag, nullptr, b.Y, k,
+                                                SolvePlanes{b.pa, ldk, b.psa, hat, ldr, b.ce_ps});
+  RET(cudaGetLastError());
+  // pass 2 to first order: G = U1^T U1 = I + E, U2 = U1 (I - Phi(E)^T)
+  RET(tc_partials(H, H, k, k, rows, &sp, b, st));
+  note_launch();
+  const unsigned kt = (unsigned)((ldk + 31) / 32);
+  cholqr_linear_kernel<<<dim3(kt, kt), 256, 0, st>>>(b.part, sp, k, CQ_LINEAR_EMAX, G, b.pb, ldk,
+                                                     b.psb, need_full);
+  RET(cudaGetLastError());
+  // the full second pass, only if E was too large: U1 -> b.Q
+  note_launch();
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 0.25f, 0, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+                                       need_full);
+  RET(cudaGetLastError());
+  note_launch();
+  cholqr_solve<<<sgrid, CQ_SOLVE_NT, ssm, st>>>(b.Y, k, rows, k, b.chol_L, b.chol_d, b.chol_li,
+                                                b.chol_flag, need_full, b.Q, k, SolvePlanes{});
+  RET(cudaGetLastError());
+  // a breakdown in either pass: block Gram-Schmidt on Y (the input, or U1
+  // after a breakdown of the second pass)
+  RET(block_cgs(b.Y, rows, k, b, st, b.chol_flag));
+  RET(tc_partials(plane_op(b.pa, rows, k, ldk, b.psa), plane_op(b.pb, k, k, ldk, b.psb), rows, k, k,
+                  &sp, b, st));
+  // the basis: FP64 factor (U, or V transposed) and planes of its transpose
+  note_launch();
+  basis_kernel<<<bgrid, 256, 0, st>>>(BasisSrc{b.part, sp, b.Y, b.chol_flag, b.Q, need_full}, rows, k,
+                                      nullptr, 0.0, 0ull, b.seed_base, nullptr,
+                                      dir_right ? left : nullptr, dir_right ? nullptr : right, hat,
+                                      ldr, b.ce_ps);
+  RET(cudaGetLastError());
+  // centre and Gram in one product: [U^T C_E | U^T U], or [C_E V ; V^T V]
+  CentreOut o;
+  o.k = k;
+  o.dscal = b.dscal;
+  o.live = b.live;
+  o.ce_ss = b.ce_ss;
+  o.thresh = thresh;
+  o.disc_max = disc_max;
+  const TcOperand X = plane_op(cet, other + k, rows, ldr, b.ce_ps);
+  const int R = dir_right ? k : other + k, Cc = dir_right ? other + k : k;
+  RET(dir_right ? tc_partials(H, X, R, Cc, rows, &sp, b, st)
+                : tc_partials(X, H, R, Cc, rows, &sp, b, st));
+  o.out = dir_right ? right : left;
+  o.ldo = dir_right ? n : k;
+  o.r_gram = dir_right ? R : other;
+  o.c_gram = dir_right ? other : Cc;
+  note_launch();
+  centre_kernel<<<dim3((unsigned)((Cc + 31) / 32), (unsigned)((R + 31) / 32)), 256, 0, st>>>(
+      b.part, sp, R, Cc, o);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 unsigned long long g_orth_cluster_calls = 0;
@@ -1249,6 +1633,8 @@ thread_local unsigned long long t_orth_cluster_calls = 0;
 
 size_t subspace_plane_elems_a(int cap) { return 3 * (size_t)(4 * cap) * tc_ld(4 * cap); }
 size_t subspace_plane_elems_b(int cap) { return 3 * (size_t)(4 * cap) * tc_ld(4 * cap); }
+// C_E's planes with room for the basis' transpose behind them
+size_t subspace_plane_elems_ce(int cap) { return 3 * (size_t)(5 * cap) * tc_ld(4 * cap); }
 
 namespace {
 // max over live columns of |Q^T Q - I| (dead columns, norm < 1/2, are skipped)
@@ -1348,11 +1734,14 @@ cudaError_t subspace_split(const double* CE, int m, int n, int k, int dir_right,
                            double* disc_max, double thresh) {
   (void)CE;
   if (k > SUBSPACE_MAX_K || k > m || k > n) return cudaErrorInvalidValue;
+  if (k <= b.orth_block)
+    return narrow_split(m, n, k, dir_right, warm, kold, left, right, seed, b, st, disc_max, thresh);
   const double inv_mn = 1.0 / ((double)m * n);
   const long long ldn = tc_ld(n), ldm = tc_ld(m);
   const View ce = planes_view(b.ce_rm, ldn, b.ce_ps);    // C_E   (m rows, K = n)
   const View cet = planes_view(b.ce_tr, ldm, b.ce_ps);   // C_E^T (n rows, K = m)
-  RET(cudaMemsetAsync(b.dscal + 1, 0, 2 * sizeof(double), st));
+  RET(cudaMemsetAsync(b.zero, 0, b.zero_words * sizeof(int), st));
+  RET(cudaMemsetAsync(b.chol_flag, 0, sizeof(int), st));
   if (dir_right) {
     // warm start: rows of the current C_{i+1} (kold x n) -> Q (n x k)
     note_launch();
@@ -1364,8 +1753,8 @@ cudaError_t subspace_split(const double* CE, int m, int n, int k, int dir_right,
     add_noise_kernel<<<grid_for((long long)m * k), 256, 0, st>>>(b.Y, (long long)m * k, b.ce_ss,
                                                                  inv_mn, seed + 7, b.seed_base);
     RET(cudaGetLastError());
-    float* U = nullptr;
-    RET(orthonormalise(b.Y, m, k, b, st, &U));
+    float* U = b.Y;
+    RET(orthonormalise_blocks(U, m, k, b, st));
     RET(orth_check(U, m, k, b, st));
     RET(split_guard(k, b, st));
     // C_i = U (m x k); C_{i+1} = U^T C_E (k x n)
@@ -1387,8 +1776,8 @@ cudaError_t subspace_split(const double* CE, int m, int n, int k, int dir_right,
     add_noise_kernel<<<grid_for((long long)n * k), 256, 0, st>>>(b.Y, (long long)n * k, b.ce_ss,
                                                                  inv_mn, seed + 7, b.seed_base);
     RET(cudaGetLastError());
-    float* V = nullptr;
-    RET(orthonormalise(b.Y, n, k, b, st, &V));
+    float* V = b.Y;
+    RET(orthonormalise_blocks(V, n, k, b, st));
     RET(orth_check(V, n, k, b, st));
     RET(split_guard(k, b, st));
     // C_{i+1} = V^T (k x n); C_i = C_E V (m x k)
@@ -1412,5 +1801,13 @@ cudaError_t subspace_split(const double* CE, int m, int n, int k, int dir_right,
     split_finish_kernel<<<1, 1, 0, st>>>(b.ce_ss, b.dscal, thresh, disc_max);
     RET(cudaGetLastError());
   }
-  return cudaSuccess;
+  return cudaMemsetAsync(b.ce_ss, 0, sizeof(double), st);
+}
+
+const __nv_bfloat16* subspace_basis_planes(const SubspaceBuffers& b, int m, int n, int k,
+                                           int dir_right, long long* ld, long long* ps) {
+  if (k > b.orth_block || k > SUBSPACE_MAX_K) return nullptr;
+  *ld = tc_ld(dir_right ? m : n);
+  *ps = b.ce_ps;
+  return dir_right ? b.ce_tr + (long long)n * *ld : b.ce_rm + (long long)m * *ld;
 }

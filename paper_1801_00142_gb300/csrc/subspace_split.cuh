@@ -21,11 +21,17 @@ struct SubspaceBuffers {
   long long psa, psb;  // their plane strides
   int* err;            // bounded-wait error flag of the tensor-core GEMM
   // C_E as BF16 planes in both orientations and its squared Frobenius norm,
-  // written by reduce_partials_planes before subspace_split reads them
-  __nv_bfloat16* ce_rm;   // [plane][m][tc_ld(n)]
-  __nv_bfloat16* ce_tr;   // [plane][n][tc_ld(m)]
+  // written by reduce_partials_planes before subspace_split reads them; the
+  // split puts the transposed basis behind the rows of one of them
+  __nv_bfloat16* ce_rm;   // [plane][m (+ k)][tc_ld(n)]
+  __nv_bfloat16* ce_tr;   // [plane][n (+ k)][tc_ld(m)]
   long long ce_ps;        // plane stride of both (elements)
-  double* ce_ss;          // ||C_E||_F^2 (device scalar)
+  double* ce_ss;          // ||C_E||_F^2 (device scalar); the split leaves it at zero
+  // words the split clears before anything else: dscal, live, and whatever the
+  // exact fallback after it wants cleared
+  int* zero;
+  int zero_words;         // at most 64
+  int* live;              // [0] a live column seen, [1] CTAs finished (centre_kernel)
   // scaled CholeskyQR2: packed Cholesky factor, column scaling, 1 / L_jj,
   // breakdown flag (0: the fast path succeeded)
   float* chol_L;          // w (w + 1) / 2 for a column block of width w
@@ -56,6 +62,8 @@ extern thread_local unsigned long long t_orth_cluster_calls;
 // BF16 elements of pa and pb for bond capacity cap.
 size_t subspace_plane_elems_a(int cap);
 size_t subspace_plane_elems_b(int cap);
+// ... and of ce_rm and of ce_tr.
+size_t subspace_plane_elems_ce(int cap);
 
 // Floats needed by the float buffers above for bond capacity cap (m, n <= 4 cap).
 size_t subspace_buffer_floats(int cap);
@@ -78,6 +86,11 @@ cudaError_t subspace_split(const double* CE, int m, int n, int k, int dir_right,
                            unsigned long long seed, const SubspaceBuffers& b, cudaStream_t st,
                            double* disc_max, double thresh);
 const double* subspace_defect(const SubspaceBuffers& b);
+// BF16 planes (3, row stride *ld, plane stride *ps) of the transposed
+// orthonormal factor that subspace_split(m, n, k, dir_right) left behind, valid
+// unless the exact fallback replaced it; null if that split leaves none.
+const __nv_bfloat16* subspace_basis_planes(const SubspaceBuffers& b, int m, int n, int k,
+                                           int dir_right, long long* ld, long long* ps);
 // Advance the device seed counter (once per product, inside a captured graph
 // too, so that every doubling draws fresh noise).
 cudaError_t subspace_next_seed(const SubspaceBuffers& b, cudaStream_t st);

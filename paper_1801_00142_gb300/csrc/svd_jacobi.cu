@@ -639,7 +639,8 @@ SvdSetup svd_setup() {
 
 cudaError_t svd_launch(const double* M, int m, int n, int kcap, double rel_tol, SplitMode mode,
                        double* left, double* right, const SvdBuffers& buf, cudaStream_t st,
-                       const double* run_if, double thresh, const SvdDeviceAcc& acc) {
+                       const double* run_if, double thresh, const SvdDeviceAcc& acc,
+                       bool cleared = false) {
   const int p = mode == SPLIT_RIGHT ? m : n, q = mode == SPLIT_RIGHT ? n : m;
   const int rmax = p < q ? p : q;
   if (m < 1 || n < 1 || kcap < 1 || (size_t)m * n > buf.max_elems || p > buf.max_cols)
@@ -665,9 +666,11 @@ cudaError_t svd_launch(const double* M, int m, int n, int kcap, double rel_tol, 
   a.run_if = run_if;
   a.thresh = thresh;
   a.acc = acc;
-  if ((e = cudaMemsetAsync(buf.counter, 0, 8 * sizeof(int), st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(buf.kept, 0, 4 * sizeof(int), st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(buf.stats, 0, 4 * sizeof(double), st)) != cudaSuccess) return e;
+  if (!cleared) {
+    if ((e = cudaMemsetAsync(buf.counter, 0, 8 * sizeof(int), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(buf.kept, 0, 4 * sizeof(int), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(buf.stats, 0, 4 * sizeof(double), st)) != cudaSuccess) return e;
+  }
   note_launch();
   // One cluster while its SMs finish a step in about the time of a grid
   // barrier: a QR step costs 3 p q FP64 operations, 32 a clock on 16 SMs.
@@ -690,9 +693,10 @@ cudaError_t svd_launch(const double* M, int m, int n, int kcap, double rel_tol, 
 
 cudaError_t svd_split_f64_if(const double* M, int m, int n, int kcap, SplitMode mode,
                              double* left, double* right, const SvdBuffers& buf, cudaStream_t st,
-                             const double* run_if, double thresh, const SvdDeviceAcc& acc) {
+                             const double* run_if, double thresh, const SvdDeviceAcc& acc,
+                             bool cleared) {
   if (!run_if) return cudaErrorInvalidValue;
-  return svd_launch(M, m, n, kcap, 0.0, mode, left, right, buf, st, run_if, thresh, acc);
+  return svd_launch(M, m, n, kcap, 0.0, mode, left, right, buf, st, run_if, thresh, acc, cleared);
 }
 
 cudaError_t svd_split_f64(const double* M, int m, int n, int kcap, double rel_tol, SplitMode mode,

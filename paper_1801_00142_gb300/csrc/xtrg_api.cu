@@ -113,7 +113,8 @@ bool plan_sizes(int L, int DH, const xtrg_config* cfg, Plan* p) {
     mb += up(pl * p->m_ct * 2) + up(p->m_part * 4) + 2 * ALIGN;
     mb += up(subspace_buffer_floats(p->cap) * 4) + 3 * ALIGN;
     mb += up(subspace_plane_elems_a(p->cap) * 2) + up(subspace_plane_elems_b(p->cap) * 2);
-    mb += 2 * up(subspace_plane_elems_a(p->cap) * 2) + ALIGN;   // C_E planes, both orientations
+    // C_E planes, both orientations, and the scalars cleared per update
+    mb += 2 * up(subspace_plane_elems_ce(p->cap) * 2) + 2 * ALIGN;
     mb += up(SUBSPACE_CHOL_FLOATS * 4) + 2 * up(SUBSPACE_BLOCK_K * 4) + ALIGN;   // CholeskyQR2 factor
     p->mixed_bytes = (cfg->prec == XTRG_FP64) ? 0 : mb;
   }
@@ -757,18 +758,30 @@ xtrg_status mixed_right_part(xtrg_ctx* ctx, const DevMpo& C, int j) {
   return XTRG_OK;
 }
 
+// Largest orthonormality defect of the subspace truncation's factor that is
+// accepted; above it the exact FP64 split runs instead.
+constexpr double ORTH_DEFECT_MAX = 1e-4;
+
 // new environment at slot from a C site (FP64) and the Lp or Rp planes:
 //   left:  V'[c'][b'][a'] = sum_{(c,s,u)} C_i[(c,s,u)][c'] Lp[(c,s,u)][(b',a')]
 //   right: V'[c'][b'][a'] = sum_{(s',u',c'')} C_j[c'][(s',u',c'')] Rp[(s',u',c'')][(b',a')]
 xtrg_status mixed_env(xtrg_ctx* ctx, const double* Csite, int kout, int kin, bool left,
-                      const __nv_bfloat16* part, int a, int slot) {
+                      const __nv_bfloat16* part, int a, int slot,
+                      const __nv_bfloat16* basis = nullptr, long long basis_ps = 0) {
   const int P = ctx->m.P;
   const long long ab = (long long)a * a, ldP = tc_ld(ab), ldK = tc_ld(kin), ldE = tc_ld(a);
-  // C^T-part [c'][k]: left reads C_i[k][c'], right reads C_j[c'][k]
-  CKM(to_planes(Csite, left ? idx_plain(1) : idx_plain(kin), left ? idx_plain(kout) : idx_plain(1),
-                0, kout, kin, 1, ctx->m.Ct, ldK, 0, P, ctx->plan.m_ct, ctx->st));
-  ctx->cur_tag = 4;
+  // C^T-part [c'][k]: left reads C_i[k][c'], right reads C_j[c'][k].  The
+  // truncation has left its planes (basis) unless the exact split replaced it.
+  const Idx3 rv = left ? idx_plain(1) : idx_plain(kin), kv = left ? idx_plain(kout) : idx_plain(1);
   TcOperand Ac = opnd(ctx->m.Ct, P, kout, kin, ldK, 0, ctx->plan.m_ct, 1);
+  if (basis) {
+    Ac = opnd(basis, P, kout, kin, ldK, 0, basis_ps, 1);
+    CKM(to_planes_if(Csite, rv, kv, kout, kin, const_cast<__nv_bfloat16*>(basis), ldK, P, basis_ps,
+                     subspace_defect(ctx->m.sb), ORTH_DEFECT_MAX, ctx->st));
+  } else {
+    CKM(to_planes(Csite, rv, kv, 0, kout, kin, 1, ctx->m.Ct, ldK, 0, P, ctx->plan.m_ct, ctx->st));
+  }
+  ctx->cur_tag = 4;
   // B(n = (b',a'), k = (c,s,u)) is the half itself, [k][n] with row stride
   // ldP: staged MN-major, no transpose pass
   TcOperand Bt = opnd(part, P, (int)ab, kin, ldP, 0, ctx->plan.m_lp, 1);
@@ -881,10 +894,6 @@ xtrg_status mixed_ce(xtrg_ctx* ctx, const __nv_bfloat16* Lp, const __nv_bfloat16
   return XTRG_OK;
 }
 
-// Largest orthonormality defect of the subspace truncation's factor that is
-// accepted; above it the exact FP64 split runs instead.
-constexpr double ORTH_DEFECT_MAX = 1e-4;
-
 // The one host read of a tensor-core product: the bounded-wait flag of the
 // GEMMs, the largest discarded weight of the last sweep, the exact-split
 // fallbacks and their status.
@@ -919,6 +928,7 @@ xtrg_status compress_mixed(xtrg_ctx* ctx, DevMpo& C, int dstar, int sweeps) {
   // the end of the product
   CKM(cudaMemsetAsync(ctx->m.err, 0, sizeof(int), ctx->st));
   CKM(cudaMemsetAsync(ctx->m.acc + 3, 0, sizeof(double), ctx->st));
+  CKM(cudaMemsetAsync(ctx->m.sb.ce_ss, 0, sizeof(double), ctx->st));   // each split clears it again
   CKM(subspace_next_seed(ctx->m.sb, ctx->st));
   TRY(mixed_unit_env(ctx, 0));
   TRY(mixed_unit_env(ctx, L));
@@ -950,7 +960,11 @@ xtrg_status compress_mixed(xtrg_ctx* ctx, DevMpo& C, int dstar, int sweeps) {
         if (ctx->profiling) TRY(ev_pair(ctx, TAG_SPLIT, &s0, &s1));
         const SplitMode mode = dir == 0 ? SPLIT_RIGHT : SPLIT_LEFT;
         const SvdDeviceAcc a{last ? acc.disc_max : nullptr, acc.runs, acc.status};
+        long long bld = 0, bps = 0;
+        const __nv_bfloat16* basis =
+            subspace_basis_planes(ctx->m.sb, m, n, k, dir == 0 ? 1 : 0, &bld, &bps);
         if (k > SUBSPACE_MAX_K) {
+          CKM(cudaMemsetAsync(ctx->m.sb.ce_ss, 0, sizeof(double), ctx->st));
           // wider than the blocked orthonormalisation handles: exact split
           CKM(svd_split_f64_if(ctx->CE, m, n, k, mode, C.site[i], C.site[i + 1], ctx->svd, ctx->st,
                                ctx->m.acc + 2, 0.0, a));
@@ -965,7 +979,7 @@ xtrg_status compress_mixed(xtrg_ctx* ctx, DevMpo& C, int dstar, int sweeps) {
           // deficient spectrum): the exact FP64 Jacobi split replaces it,
           // decided on the device from the defect
           CKM(svd_split_f64_if(ctx->CE, m, n, k, mode, C.site[i], C.site[i + 1], ctx->svd, ctx->st,
-                               subspace_defect(ctx->m.sb), ORTH_DEFECT_MAX, a));
+                               subspace_defect(ctx->m.sb), ORTH_DEFECT_MAX, a, true));
         }
         if (s1) CKM(cudaEventRecord(s1, ctx->st));
         C.dims[i + 1] = k;
@@ -973,9 +987,10 @@ xtrg_status compress_mixed(xtrg_ctx* ctx, DevMpo& C, int dstar, int sweeps) {
         TRY(debug_check(ctx, "right factor", C.site[i + 1], (long long)k * n, i));
         ctx->flops_split += 2.0 * m * (double)n * k * 2 + 3.0 * (2.0 * (dir == 0 ? m : n) * k * k);
         if (dir == 0)
-          TRY(mixed_env(ctx, C.site[i], k, m, true, ctx->m.lpc[i], R.dims[i + 1], i + 1));
+          TRY(mixed_env(ctx, C.site[i], k, m, true, ctx->m.lpc[i], R.dims[i + 1], i + 1, basis, bps));
         else
-          TRY(mixed_env(ctx, C.site[i + 1], k, n, false, ctx->m.rpc[i + 1], R.dims[i + 1], i + 1));
+          TRY(mixed_env(ctx, C.site[i + 1], k, n, false, ctx->m.rpc[i + 1], R.dims[i + 1], i + 1, basis,
+                        bps));
         ctx->updates++;
       }
     }
@@ -1208,15 +1223,29 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
       }
       ctx->m.sb.orth_bar = (unsigned*)carve(ctx, 16);
       ok = ok && ctx->m.sb.orth_bar;
-      ctx->m.sb.dscal = (double*)carve(ctx, 16);
+      // scalars that every truncation clears in one go: its own, then the
+      // exact split's
+      {
+        char* z = carve(ctx, 192);
+        ok = ok && z;
+        if (z) {
+          ctx->m.sb.zero = (int*)z;
+          ctx->m.sb.zero_words = 48;
+          ctx->m.sb.dscal = (double*)z;             // 4 doubles
+          ctx->m.sb.live = (int*)(z + 32);          // 2 ints
+          ctx->svd.counter = (int*)(z + 64);        // 8 ints
+          ctx->svd.kept = (int*)(z + 96);           // 4 ints
+          ctx->svd.stats = (double*)(z + 128);      // 8 doubles
+        }
+      }
       ctx->m.sb.pa = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_a(p.cap) * 2);
       ctx->m.sb.pb = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_b(p.cap) * 2);
       ctx->m.sb.psa = (long long)(subspace_plane_elems_a(p.cap) / 3);
       ctx->m.sb.psb = (long long)(subspace_plane_elems_b(p.cap) / 3);
       ctx->m.sb.err = ctx->m.err;
-      ctx->m.sb.ce_ps = (long long)(subspace_plane_elems_a(p.cap) / 3);
-      ctx->m.sb.ce_rm = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_a(p.cap) * 2);
-      ctx->m.sb.ce_tr = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_a(p.cap) * 2);
+      ctx->m.sb.ce_ps = (long long)(subspace_plane_elems_ce(p.cap) / 3);
+      ctx->m.sb.ce_rm = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_ce(p.cap) * 2);
+      ctx->m.sb.ce_tr = (__nv_bfloat16*)carve(ctx, subspace_plane_elems_ce(p.cap) * 2);
       ctx->m.sb.ce_ss = (double*)carve(ctx, 16);
       ctx->m.sb.chol_L = (float*)carve(ctx, SUBSPACE_CHOL_FLOATS * 4);
       ctx->m.sb.chol_d = (float*)carve(ctx, SUBSPACE_BLOCK_K * 4);
