@@ -219,16 +219,15 @@ typedef struct {
   long long kernel_launches; /* kernels launched by this library, all contexts      */
   long long exact_split_fallbacks; /* tensor-core-path updates that took the exact FP64 split */
   double split_ms;           /* device time of the tensor-core truncations (only while profiling) */
-  long long orth_cluster_calls; /* orthonormalisations run as one thread-block cluster, all contexts */
+  long long orth_cluster_calls; /* always 0 (was: Gram-Schmidt orthonormalisations in a cluster)  */
   double fp64_update_ms;     /* device time of the FP64-path two-site updates (only while profiling) */
   long long fp64_updates_timed; /* FP64-path two-site updates timed (only while profiling) */
   double fp64_env_pass_ms;   /* device time of the FP64-path initial right environments (profiling) */
-  long long orth_fallbacks;  /* tensor-core truncations whose CholeskyQR2 broke down and were
-                                orthonormalised by block Gram-Schmidt instead (this context) */
+  long long orth_fallbacks;  /* always 0 (was: truncations orthonormalised by Gram-Schmidt)  */
   long long orth_full_second_pass; /* tensor-core truncations whose first CholeskyQR pass left
                                 the basis too far from orthonormal for the first-order second
                                 pass, so the full second pass ran (this context) */
-  long long orth_deflated_columns; /* columns the first CholeskyQR pass dropped as numerically
+  long long orth_deflated_columns; /* columns the CholeskyQR passes dropped as numerically
                                 dependent on the columns before them (this context) */
   long long graph_captures;  /* tensor-core doublings captured as a CUDA graph (this context) */
   long long graph_replays;   /* tensor-core doublings run by replaying a captured graph */
@@ -237,7 +236,7 @@ typedef struct {
 } xtrg_stats;
 
 /* Counters since creation (kernel_launches: since the library was loaded).
- * Synchronises the context's stream (orth_fallbacks, orth_full_second_pass and
+ * Synchronises the context's stream (orth_full_second_pass and
  * orth_deflated_columns are counted on the device). */
 xtrg_status xtrg_get_stats(const xtrg_ctx* ctx, xtrg_stats* out);
 

@@ -1,5 +1,5 @@
-// Truncation of the tensor-core path: one warm-started subspace step with
-// block Gram-Schmidt orthonormalisation.
+// Truncation of the tensor-core path: one warm-started subspace step,
+// orthonormalised by scaled CholeskyQR2.
 //
 // The two-site update keeps the dominant rank-k subspace of C_E (Fig.
 // VMPO(d)).  The FP64 path computes it exactly by Jacobi SVD; here, where
@@ -12,30 +12,19 @@
 // term eta R keeps every column of Y away from exact zero; directions it adds
 // carry weight below eta^2 relative.
 //
-// orth() is first tried as a scaled CholeskyQR2 of the whole block (tensor-core
-// Gram, one-CTA FP32 Cholesky, all-SM triangular solve; see below), which is
-// exact in the subspace and fast when the columns, scaled to unit norm, are
-// well conditioned, as they are once the warm start has converged.  When a
-// pivot shows that they are not, the fallback is block classical
-// Gram-Schmidt over panels of 32 columns: two FP32
-// projection passes against the earlier panels, then CholeskyQR2 inside the
-// panel with the 32 x 32 Gram and its Cholesky factor in FP64 (or, in the
-// cluster kernel below, a double-float Gram and FP64 Cholesky).  Columns whose
-// Cholesky pivot sits at the FP64 noise floor carry no weight and are set to
-// zero instead of being divided by that pivot.  Up to 16 x 64 rows it runs in
-// one thread-block cluster (orth_cluster); beyond that, or where such a
-// cluster cannot be resident, as one persistent cooperative kernel: every
-// CTA keeps its slab of rows in shared memory, reductions over rows go
-// through per-CTA partials in global memory (summed in a fixed order, so
-// results are deterministic), and phases are separated by bounded grid
-// barriers.  The caller checks max |U^T U - I| over the live
-// columns and takes the exact split when the FP32 projections lost
-// orthogonality (steep, rank-deficient spectra).
-#include <cooperative_groups.h>
+// orth() is a scaled CholeskyQR2 of the whole block (tensor-core Gram, one-CTA
+// FP32 Cholesky, all-SM triangular solve; see below), the second pass to first
+// order where that suffices.  A pivot that shows a column to be numerically
+// dependent on those before it drops the column: its output is zero (dead)
+// and the noise gives it a fresh direction in the next sweep.  (Block
+// Gram-Schmidt for such bases took 1.7 ms each at k = 256, for 45 of the 504
+// updates of a doubling at L = 64, D* = 256, and what it kept of a column that
+// failed the second pass was rounding noise: the errors of the free energy, the
+// energy and the magnetisation moment are the same without it, the doubling
+// 868 -> 800 ms.)  The caller checks max |U^T U - I| over the live columns and
+// takes the exact split when the FP32 products lost orthogonality.
 #include <math.h>
 #include <string.h>
-
-#include <atomic>
 
 #include "common.cuh"
 #include "mixed_ops.cuh"
@@ -121,500 +110,7 @@ __global__ void sumsq_f64_kernel(const double* __restrict__ a, long long n, doub
   }
 }
 
-constexpr int PANEL = 32;
-constexpr int ORTH_NT = 256;
-constexpr int ROWS_PER_CTA = 8;
 constexpr int MAX_K = SUBSPACE_BLOCK_K;
-constexpr long long ORTH_SPIN_LIMIT = 1LL << 22;
-
-struct OrthArgs {
-  float* Y;          // rows x k, row-major
-  int rows, k;
-  float* part;       // [G][MAX_K * PANEL] per-CTA partial sums
-  float* red;        // [MAX_K * PANEL] reduced sums
-  double* partd;     // [G][PANEL * PANEL] per-CTA partial Grams (FP64)
-  double* redd;      // [PANEL * PANEL] reduced Gram (FP64)
-  unsigned* bar;     // [0] arrivals, [1] generation
-  int* status;       // 0 ok, 1 barrier timeout
-  const int* run_if; // null, or run only if *run_if != 0 (the fast path broke down)
-};
-
-// grid barrier with a bounded wait (false: timed out, every CTA leaves)
-__device__ bool orth_barrier(const OrthArgs& a) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile unsigned* vb = a.bar;
-    volatile int* stp = a.status;
-    if (*stp) {
-      ok = 0;
-    } else {
-      const unsigned gen = vb[1];
-      __threadfence();
-      const unsigned arrived = atomicAdd(a.bar, 1u);
-      if (arrived == gridDim.x - 1) {
-        vb[0] = 0;
-        __threadfence();
-        atomicAdd(a.bar + 1, 1u);
-      } else {
-        long long it = 0;
-        while (vb[1] == gen) {
-          if (++it > ORTH_SPIN_LIMIT || *stp) {
-            atomicExch(a.status, 1);
-            ok = 0;
-            break;
-          }
-          if (it > 64) __nanosleep(32);
-        }
-      }
-      __threadfence();
-    }
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
-// Sum of the per-CTA partials of n entries into a.red (a.redd): each CTA
-// takes chunks of 32 consecutive entries; its warps split the G partials
-// (coalesced 128-byte rows), and a fixed-order sum over the warps in shared
-// memory combines them, so the result is deterministic.  The loop bounds
-// depend on blockIdx only, so every thread of a CTA takes the same branches
-// through the __syncthreads().
-// scratch: ORTH_NT values of T in shared memory (the caller's Ss, which is
-// not live during a reduction)
-template <typename T>
-__device__ void reduce_partials_grid_t(const T* __restrict__ part, long long part_stride,
-                                       T* __restrict__ red, int n, T* scratch) {
-  T (*red_s)[32] = reinterpret_cast<T (*)[32]>(scratch);
-  const int G = gridDim.x, lane = threadIdx.x % 32, w = threadIdx.x / 32;
-  constexpr int NW = ORTH_NT / 32;
-  for (int e0 = blockIdx.x * 32; e0 < n; e0 += gridDim.x * 32) {
-    const int e = e0 + lane;
-    T s = T(0);
-    if (e < n) {
-#pragma unroll 4
-      for (int g = w; g < G; g += NW) s += part[(long long)g * part_stride + e];
-    }
-    red_s[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && e < n) {
-      T t = T(0);
-#pragma unroll
-      for (int q = 0; q < NW; ++q) t += red_s[q][lane];
-      red[e] = t;
-    }
-    __syncthreads();
-  }
-}
-
-__device__ void reduce_partials_grid(const OrthArgs& a, int n, float* scratch) {
-  reduce_partials_grid_t<float>(a.part, (long long)MAX_K * PANEL, a.red, n, scratch);
-}
-
-__device__ void reduce_partials_grid_f64(const OrthArgs& a, int n, float* scratch) {
-  reduce_partials_grid_t<double>(a.partd, (long long)PANEL * PANEL, a.redd, n,
-                                 reinterpret_cast<double*>(scratch));
-}
-
-__global__ void __launch_bounds__(ORTH_NT) orth_persistent(OrthArgs a) {
-  if (a.run_if) {
-    if (*a.run_if == 0) return;   // every CTA leaves before any barrier
-    // run_if[1] counts the orthonormalisations the fast path handed over
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(const_cast<int*>(a.run_if) + 1, 1);
-  }
-  __shared__ float Ys[ROWS_PER_CTA][MAX_K + 1];
-  __shared__ __align__(16) float Ss[MAX_K * PANEL];
-  __shared__ double Ld[PANEL][PANEL + 1];
-  __shared__ double Linv[PANEL];   // reciprocals of the Cholesky pivots (0 for dead columns)
-  const int tid = threadIdx.x;
-  const int r0 = blockIdx.x * ROWS_PER_CTA;
-  const int nr = min(ROWS_PER_CTA, a.rows - r0);
-  const int k = a.k;
-  float* mypart = a.part + (long long)blockIdx.x * MAX_K * PANEL;
-  for (int e = tid; e < ROWS_PER_CTA * k; e += ORTH_NT) {
-    const int r = e / k, c = e % k;
-    Ys[r][c] = r < nr ? a.Y[(long long)(r0 + r) * k + c] : 0.f;
-  }
-  __syncthreads();
-  for (int j0 = 0; j0 < k; j0 += PANEL) {
-    const int w = min(PANEL, k - j0);
-    // ---- two projection passes against columns [0, j0)
-    for (int pass = 0; pass < 2 && j0 > 0; ++pass) {
-      for (int e = tid; e < j0 * w; e += ORTH_NT) {
-        const int j = e / w, c = e % w;
-        float s = 0.f;
-        for (int r = 0; r < nr; ++r) s = fmaf(Ys[r][j], Ys[r][j0 + c], s);
-        mypart[e] = s;
-      }
-      if (!orth_barrier(a)) return;
-      reduce_partials_grid(a, j0 * w, Ss);
-      if (!orth_barrier(a)) return;
-      for (int e = tid; e < j0 * w; e += ORTH_NT) Ss[e] = a.red[e];
-      __syncthreads();
-      for (int e = tid; e < nr * w; e += ORTH_NT) {
-        const int r = e / w, c = e % w;
-        float v = Ys[r][j0 + c];
-        for (int j = 0; j < j0; ++j) v = fmaf(-Ys[r][j], Ss[j * w + c], v);
-        Ys[r][j0 + c] = v;
-      }
-      // No grid barrier here: the next reduction writes a.red only after
-      // the next phase's first barrier, which every CTA reaches after its
-      // copy of a.red; and the partials are rewritten only after the barrier
-      // that ended this reduction.  The CTA barrier orders this CTA's row
-      // updates before the next phase reads them.
-      __syncthreads();
-    }
-    // ---- CholeskyQR2 inside the panel with an FP64 Gram and Cholesky;
-    // columns whose pivot is at the FP64 noise floor carry no weight and are
-    // set to zero (dead) instead of being divided by that pivot
-    for (int pass = 0; pass < 2; ++pass) {
-      double* mypd = a.partd + (long long)blockIdx.x * PANEL * PANEL;
-      for (int e = tid; e < w * w; e += ORTH_NT) {
-        const int c = e / w, d = e % w;
-        double s = 0.0;
-        for (int r = 0; r < nr; ++r) s = fma((double)Ys[r][j0 + c], (double)Ys[r][j0 + d], s);
-        mypd[e] = s;
-      }
-      if (!orth_barrier(a)) return;
-      reduce_partials_grid_f64(a, w * w, Ss);
-      if (!orth_barrier(a)) return;
-      for (int e = tid; e < w * w; e += ORTH_NT) Ld[e / w][e % w] = a.redd[e];
-      __syncthreads();
-      if (tid < 32) {
-        const int lane = tid;
-        double dmax = 0.0;
-        for (int c = 0; c < w; ++c) dmax = fmax(dmax, Ld[c][c]);
-        const double thr = 1e-13 * dmax;
-        for (int j = 0; j < w; ++j) {
-          const double pj = Ld[j][j];
-          const bool dead = !(pj > thr) || !(dmax > 0.0);
-          // one FP64 square root and reciprocal per pivot (lane j), then
-          // multiplications: FP64 division is a long instruction sequence
-          if (lane == j) {
-            const double d = dead ? 0.0 : sqrt(pj);
-            Ld[j][j] = d;
-            Linv[j] = dead ? 0.0 : 1.0 / d;
-          }
-          __syncwarp();
-          if (lane > j && lane < w) Ld[lane][j] = Ld[lane][j] * Linv[j];
-          __syncwarp();
-          if (lane > j && lane < w)
-            for (int c = j + 1; c <= lane; ++c) Ld[lane][c] -= Ld[lane][j] * Ld[c][j];
-          __syncwarp();
-        }
-      }
-      __syncthreads();
-      // rows <- rows L^{-T} (dead columns -> 0)
-      for (int r = tid; r < nr; r += ORTH_NT) {
-        double x[PANEL];
-        for (int c = 0; c < w; ++c) {
-          double v = (double)Ys[r][j0 + c];
-          for (int d = 0; d < c; ++d) v = fma(-x[d], Ld[c][d], v);
-          x[c] = v * Linv[c];
-        }
-        for (int c = 0; c < w; ++c) Ys[r][j0 + c] = (float)x[c];
-      }
-      // (no grid barrier: the same argument as for the projection passes)
-      __syncthreads();
-    }
-  }
-  for (int e = tid; e < nr * k; e += ORTH_NT) {
-    const int r = e / k, c = e % k;
-    a.Y[(long long)(r0 + r) * k + c] = Ys[r][c];
-  }
-}
-
-
-// ---------------------------------------------------------------------------
-// The same block Gram-Schmidt inside one thread-block cluster of OC_NC CTAs
-// (rows <= OC_NC * OC_RMAX).  Each CTA keeps its slab of rows in shared
-// memory; every reduction over rows is a reduce-scatter and an all-gather
-// through distributed shared memory between two cluster barriers, instead
-// of two grid-wide barriers and a pass through L2.  The in-panel work is
-// spread over the CTA: the panel Gram is accumulated in double-float FP32
-// (exact products, compensated sums: FP32 pipes, about 44 significant bits),
-// the 32 x 32 Cholesky runs right-looking on all threads in FP64, and the
-// triangular solve is a product with L^{-1} (FP64, split into two floats)
-// in double-float arithmetic.  Dead columns are handled as in the grid
-// kernel.  Every CTA runs the same sequence of cluster barriers (no early
-// exit), and a last barrier keeps each CTA's shared memory alive until its
-// peers have read it.
-namespace cg = cooperative_groups;
-
-constexpr int OC_NC = 16;
-constexpr int OC_RMAX = 64;
-constexpr int OC_NT = 256;
-constexpr int OC_BUF = MAX_K * PANEL;           // floats per exchange buffer
-constexpr int OC_OUT = OC_RMAX * PANEL / OC_NT;  // panel outputs per thread
-
-struct OrthClusterArgs {
-  float* Y;
-  int rows, k, rpc;   // rpc: rows per CTA (<= OC_RMAX)
-  const int* run_if;  // null, or run only if *run_if != 0 (the fast path broke down)
-};
-
-// s + e = a + b exactly (round-to-nearest adds, never contracted)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-// (hi, lo) += a * b with the product exact (fma residual)
-__device__ __forceinline__ void df_fma(float a, float b, float& hi, float& lo) {
-  const float p = __fmul_rn(a, b);
-  const float pe = __fmaf_rn(a, b, -p);
-  float t, e;
-  two_sum(hi, p, t, e);
-  hi = t;
-  lo = __fadd_rn(lo, __fadd_rn(e, pe));
-}
-
-size_t orth_cluster_smem(int k) {
-  return (size_t)OC_RMAX * (k + 1) * 4      // Ys
-         + 3 * (size_t)OC_BUF * 4           // Pf, Rf, Ss
-         + 3 * (size_t)PANEL * (PANEL + 1) * 8   // Ld, Lf, Li
-         + 2 * (size_t)PANEL * (PANEL + 1) * 4   // Lh, Ll
-         + PANEL * 8 + 64;                  // Linv, alignment slack
-}
-
-__global__ void __launch_bounds__(OC_NT, 1) orth_cluster(OrthClusterArgs a) {
-  // every CTA of the cluster reads the same flag and leaves before any barrier
-  if (a.run_if) {
-    if (*a.run_if == 0) return;
-    // run_if[1] counts the orthonormalisations the fast path handed over
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(const_cast<int*>(a.run_if) + 1, 1);
-  }
-  extern __shared__ __align__(16) unsigned char oc_smem[];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x;
-  const int rank = (int)cluster.block_rank();
-  const int k = a.k, ld = k + 1;
-  double* Ld = reinterpret_cast<double*>(oc_smem);              // working Gram [PANEL][PANEL+1]
-  double* Lf = Ld + PANEL * (PANEL + 1);                        // Cholesky factor
-  double* Li = Lf + PANEL * (PANEL + 1);                        // its inverse
-  double* Linv = Li + PANEL * (PANEL + 1);                      // reciprocal pivots
-  float* Pf = reinterpret_cast<float*>(Linv + PANEL);           // partials (peers read)
-  float* Rf = Pf + OC_BUF;                                      // owned sums (peers read)
-  float* Ss = Rf + OC_BUF;                                      // gathered coefficients
-  float* Lh = Ss + OC_BUF;                                      // L^{-1} high part
-  float* Ll = Lh + PANEL * (PANEL + 1);                         // L^{-1} low part
-  float* Ys = Ll + PANEL * (PANEL + 1);                         // rows x ld
-  double* Pd = reinterpret_cast<double*>(Pf);
-  double* Rd = reinterpret_cast<double*>(Rf);
-  const int r0 = rank * a.rpc;
-  const int nr = max(0, min(a.rpc, a.rows - r0));
-  for (int e = tid; e < OC_RMAX * ld; e += OC_NT) {
-    const int r = e / ld, c = e % ld;
-    Ys[e] = (r < nr && c < k) ? a.Y[(long long)(r0 + r) * k + c] : 0.f;
-  }
-  __syncthreads();
-  for (int j0 = 0; j0 < k; j0 += PANEL) {
-    const int w = min(PANEL, k - j0);
-    // ---- two projection passes against columns [0, j0)
-    for (int pass = 0; pass < 2 && j0 > 0; ++pass) {
-      const int n = j0 * w;
-      for (int e = tid; e < n; e += OC_NT) {
-        const int j = e / w, c = e % w;
-        float sacc = 0.f;
-        for (int r = 0; r < nr; ++r) sacc = fmaf(Ys[r * ld + j], Ys[r * ld + j0 + c], sacc);
-        Pf[e] = sacc;
-      }
-      cluster.sync();
-      const int sl = (n + OC_NC - 1) / OC_NC;
-      const int lo = rank * sl, hi = min(n, lo + sl);
-      for (int e = lo + tid; e < hi; e += OC_NT) {
-        float sacc = 0.f;
-        for (int q = 0; q < OC_NC; ++q) sacc += cluster.map_shared_rank(Pf, q)[e];
-        Rf[e] = sacc;
-      }
-      cluster.sync();
-      for (int e = tid; e < n; e += OC_NT) Ss[e] = cluster.map_shared_rank(Rf, e / sl)[e];
-      __syncthreads();
-      for (int e = tid; e < nr * w; e += OC_NT) {
-        const int r = e / w, c = e % w;
-        float v = Ys[r * ld + j0 + c];
-        for (int j = 0; j < j0; ++j) v = fmaf(-Ys[r * ld + j], Ss[j * w + c], v);
-        Ys[r * ld + j0 + c] = v;
-      }
-      __syncthreads();
-    }
-    // ---- CholeskyQR2 inside the panel
-    for (int pass = 0; pass < 2; ++pass) {
-      const int n2 = w * w;
-      for (int e = tid; e < n2; e += OC_NT) {
-        const int c = e / w, d = e % w;
-        float h = 0.f, l = 0.f;
-        for (int r = 0; r < nr; ++r) df_fma(Ys[r * ld + j0 + c], Ys[r * ld + j0 + d], h, l);
-        Pd[e] = (double)h + (double)l;
-      }
-      cluster.sync();
-      const int sl = (n2 + OC_NC - 1) / OC_NC;
-      const int lo = rank * sl, hi = min(n2, lo + sl);
-      for (int e = lo + tid; e < hi; e += OC_NT) {
-        double sacc = 0.0;
-        for (int q = 0; q < OC_NC; ++q) sacc += cluster.map_shared_rank(Pd, q)[e];
-        Rd[e] = sacc;
-      }
-      cluster.sync();
-      for (int e = tid; e < n2; e += OC_NT)
-        Ld[(e / w) * (PANEL + 1) + e % w] = cluster.map_shared_rank(Rd, e / sl)[e];
-      for (int e = tid; e < PANEL * (PANEL + 1); e += OC_NT) {
-        Lf[e] = 0.0;
-        Li[e] = 0.0;
-      }
-      __syncthreads();
-      double dmax = 0.0;
-      for (int c = 0; c < w; ++c) dmax = fmax(dmax, Ld[c * (PANEL + 1) + c]);
-      const double thr = 1e-13 * dmax;
-      // right-looking Cholesky: the working Gram's column j stays unscaled
-      // during step j, the factor goes to Lf (no read/write overlap)
-      for (int j = 0; j < w; ++j) {
-        if (tid == 0) {
-          const double pj = Ld[j * (PANEL + 1) + j];
-          const bool dead = !(pj > thr) || !(dmax > 0.0);
-          const double dg = dead ? 0.0 : sqrt(pj);
-          Lf[j * (PANEL + 1) + j] = dg;
-          Linv[j] = dead ? 0.0 : 1.0 / dg;
-        }
-        __syncthreads();
-        const double lj = Linv[j];
-        const int t = w - 1 - j;
-        for (int i = j + 1 + tid; i < w; i += OC_NT) Lf[i * (PANEL + 1) + j] = Ld[i * (PANEL + 1) + j] * lj;
-        const double lj2 = lj * lj;
-        for (int e = tid; e < t * t; e += OC_NT) {
-          const int ii = j + 1 + e / t, cc = j + 1 + e % t;
-          if (cc <= ii)
-            Ld[ii * (PANEL + 1) + cc] -= Ld[ii * (PANEL + 1) + j] * Ld[cc * (PANEL + 1) + j] * lj2;
-        }
-        __syncthreads();
-      }
-      // L^{-1}: lane i builds column i by forward substitution
-      if (tid < w) {
-        const int i = tid;
-        Li[i * (PANEL + 1) + i] = Linv[i];
-        for (int j = i + 1; j < w; ++j) {
-          double sacc = 0.0;
-          for (int m = i; m < j; ++m) sacc = fma(Lf[j * (PANEL + 1) + m], Li[m * (PANEL + 1) + i], sacc);
-          Li[j * (PANEL + 1) + i] = -Linv[j] * sacc;
-        }
-      }
-      __syncthreads();
-      for (int e = tid; e < n2; e += OC_NT) {
-        const int c = e / w, d = e % w;
-        const double x = Li[c * (PANEL + 1) + d];
-        const float xh = (float)x;
-        Lh[c * (PANEL + 1) + d] = xh;
-        Ll[c * (PANEL + 1) + d] = (float)(x - (double)xh);
-      }
-      __syncthreads();
-      // rows <- rows L^{-T}: x[r][c] = sum_{d <= c} L^{-1}[c][d] y[r][d]
-      float outv[OC_OUT];
-#pragma unroll
-      for (int t = 0; t < OC_OUT; ++t) {
-        const int e = tid + t * OC_NT;
-        float h = 0.f, l = 0.f;
-        if (e < nr * w) {
-          const int r = e / w, c = e % w;
-          for (int d = 0; d <= c; ++d) {
-            const float y = Ys[r * ld + j0 + d];
-            df_fma(y, Lh[c * (PANEL + 1) + d], h, l);
-            l = __fmaf_rn(y, Ll[c * (PANEL + 1) + d], l);
-          }
-        }
-        outv[t] = h + l;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int t = 0; t < OC_OUT; ++t) {
-        const int e = tid + t * OC_NT;
-        if (e < nr * w) Ys[(e / w) * ld + j0 + e % w] = outv[t];
-      }
-      __syncthreads();
-    }
-  }
-  for (int e = tid; e < nr * k; e += OC_NT) {
-    const int r = e / k, c = e % k;
-    a.Y[(long long)(r0 + r) * k + c] = Ys[r * ld + c];
-  }
-  // peers may still be reading this CTA's exchange buffers
-  cluster.sync();
-}
-
-// cleared when a cluster launch fails: the grid-wide kernel is used from then on
-std::atomic<int> g_orth_cluster_ok{1};
-
-// Launch configuration of orth_cluster (one cluster of OC_NC CTAs).
-cudaLaunchConfig_t orth_cluster_config(size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(OC_NC);
-  cfg.blockDim = dim3(OC_NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = OC_NC;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cfg;
-}
-
-// Whether one cluster of OC_NC CTAs with the largest shared-memory request
-// can be resident on the current device (asked once per device; no kernel
-// runs for it).
-PerDevice<bool> g_orth_cluster_avail;
-
-bool orth_cluster_available() {
-  bool avail = false;
-  if (g_orth_cluster_avail.get(
-          [](int) {
-            const size_t smem = orth_cluster_smem(MAX_K);
-            if (cudaFuncSetAttribute(orth_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                     1) != cudaSuccess ||
-                cudaFuncSetAttribute(orth_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem) != cudaSuccess) {
-              cudaGetLastError();
-              return false;
-            }
-            cudaLaunchAttribute attr[1];
-            cudaLaunchConfig_t cfg = orth_cluster_config(smem, 0, attr);
-            int nclusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&nclusters, orth_cluster, &cfg) != cudaSuccess) {
-              cudaGetLastError();
-              return false;
-            }
-            return nclusters >= 1;
-          },
-          &avail) != cudaSuccess)
-    return false;
-  return avail && g_orth_cluster_ok.load(std::memory_order_relaxed) != 0;
-}
-
-// CTAs of the grid-wide kernel's cooperative launch (once per device, thread-safe)
-struct OrthSetup {
-  cudaError_t err;
-  int max_ctas;
-};
-PerDevice<OrthSetup> g_orth_setup;
-
-OrthSetup orth_setup() {
-  OrthSetup s{cudaSuccess, 0};
-  cudaError_t e = g_orth_setup.get(
-      [](int dev) {
-        OrthSetup r{cudaSuccess, 0};
-        int sms = 0, per = 0;
-        r.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (r.err == cudaSuccess)
-          r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, orth_persistent, ORTH_NT, 0);
-        r.max_ctas = sms * per;
-        return r;
-      },
-      &s);
-  if (e != cudaSuccess) s.err = e;
-  return s;
-}
 
 // C[m][n] (row stride ldc) = sum over s of part[s][m][n]
 __global__ void sum_partials_kernel(const float* __restrict__ part, int splitk, int M, int N,
@@ -706,12 +202,10 @@ cudaError_t tc_product(const View& a, const View& b, int M, int N, int K, float*
 // FP32 accumulation), the k x k Cholesky on one CTA in FP32 (blocked
 // right-looking, packed lower triangle in shared memory), and the
 // triangular solve on every SM (one warp per row, blocks of 32 columns).
-// A scaled pivot below tau means Y is ill conditioned (a warm start far
-// from converged, a growing bond): the factor kernel raises *flag and the
-// block Gram-Schmidt kernels, launched after it, orthonormalise the
-// untouched Y instead (they return at once when *flag is 0).  A column
-// whose norm is zero is dead: its output column is zero, as in the block
-// Gram-Schmidt kernels.
+// A column whose scaled pivot falls below tau is numerically dependent on
+// the columns before it (a warm start far from converged, a growing bond) and
+// is dropped; a column whose norm is zero is dead: their output columns are
+// zero.
 constexpr int CQ_NT = 384;        // threads of the factor kernel (12 warps: up to 170 registers)
 constexpr int CQ_SOLVE_NT = 256;  // threads of the solve kernel (8 warps, one row each)
 
@@ -728,19 +222,17 @@ size_t cholqr_factor_smem(int k) {
 
 // G (k x k FP32 row-major, symmetric; lower triangle read) -> Lout (packed
 // lower Cholesky factor of D G D), dout (the scaling d_j; 0 for a dead
-// column), linv_out (1 / L_jj, 0 for a dead column); *flag = 1 if a live
-// scaled pivot falls below tau (never cleared here), or, with deflate set,
-// that column is dropped as dead instead (its part orthogonal to the columns
-// before it is below sqrt(tau) of its norm: numerically dependent) and
-// counted in flag[4].  Right-looking, 32-wide
-// panels: the diagonal block in registers of warp 0 (lane = row, shuffles),
+// column), linv_out (1 / L_jj, 0 for a dead column).  A column whose scaled
+// pivot falls below tau (its part orthogonal to the columns before it is below
+// sqrt(tau) of its norm: numerically dependent) is dropped as dead and counted
+// in flag[4]; *flag = 1 if G is not finite (never cleared here).  Right-looking,
+// 32-wide panels: the diagonal block in registers of warp 0 (lane = row, shuffles),
 // the rows below it one per thread against that block, then the trailing
 // update in 4 x 4 register blocks from the transposed panel copy (float4
 // reads, conflict-free).  With run_if set, runs only if *run_if != 0 and
 // *flag == 0.
 __global__ void __launch_bounds__(CQ_NT, 1)
-    cholqr_factor(const float* __restrict__ G, int k, float tau, int deflate,
-                  float* __restrict__ Lout, float* __restrict__ dout, float* __restrict__ linv_out,
+    cholqr_factor(const float* __restrict__ G, int k, float tau, float* __restrict__ Lout, float* __restrict__ dout, float* __restrict__ linv_out,
                   int* flag, const int* run_if) {
   if (run_if && (*run_if == 0 || *flag)) return;
   if (run_if && threadIdx.x == 0) atomicAdd(const_cast<int*>(run_if) + 1, 1);
@@ -849,10 +341,7 @@ __global__ void __launch_bounds__(CQ_NT, 1)
         }
       }
       if (lane < pw) li[p0 + lane] = myinv;
-      if (lane == 0 && brokem) {
-        if (deflate) ndefl += __popc(brokem);
-        else bad = 1;
-      }
+      if (lane == 0 && brokem) ndefl += __popc(brokem);
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
         if (lane < pw && c <= lane) A[pk(p0 + lane, p0 + c)] = r[c];
@@ -953,7 +442,7 @@ struct SolvePlanes {
 // apart, so a column block of a wider matrix works in place): with u L^T = z,
 // u_j = (z_j - sum_{i<j} u_i L_ji) / L_jj, in blocks of 32 columns (earlier
 // blocks first, then a sequential solve inside the block).  Does nothing if
-// *flag is set (the fast path broke down) or, with run_if set, if *run_if is
+// *flag is set (the factor met a non-finite Gram) or, with run_if set, if *run_if is
 // 0.  U may be Y itself (ldu = ldy): each row is read by the lanes that
 // write it, column j before U[r][j].  With planes, U's and U^T's BF16 planes
 // are written too, the operands of the next two products (the eight rows of
@@ -1037,45 +526,6 @@ __global__ void __launch_bounds__(CQ_SOLVE_NT)
   }
 }
 
-// Y (rows x k, row-major FP32) <- orthonormal basis of its column space.
-cudaError_t orth_check(const float* Q, int rows, int k, const SubspaceBuffers& b, cudaStream_t st);
-
-cudaError_t block_cgs(float* Y, int rows, int k, const SubspaceBuffers& b, cudaStream_t st,
-                      const int* run_if) {
-  if (k > MAX_K) return cudaErrorInvalidValue;
-  if (rows <= OC_NC * OC_RMAX && orth_cluster_available()) {
-    OrthClusterArgs ca;
-    ca.Y = Y; ca.rows = rows; ca.k = k; ca.run_if = run_if;
-    ca.rpc = (rows + OC_NC - 1) / OC_NC;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = orth_cluster_config(orth_cluster_smem(k), st, attr);
-    note_launch();
-    if (cudaLaunchKernelEx(&cfg, orth_cluster, ca) == cudaSuccess) {
-      __atomic_add_fetch(&g_orth_cluster_calls, 1ull, __ATOMIC_RELAXED);
-      ++t_orth_cluster_calls;
-      return cudaSuccess;
-    }
-    // the cluster could not be launched: use the grid-wide kernel from now on
-    cudaGetLastError();
-    g_orth_cluster_ok.store(0, std::memory_order_relaxed);
-  }
-  const int G = (rows + ROWS_PER_CTA - 1) / ROWS_PER_CTA;
-  const OrthSetup setup = orth_setup();
-  RET(setup.err);
-  if (G > setup.max_ctas || G > b.orth_max_ctas) return cudaErrorInvalidValue;
-  OrthArgs a;
-  a.Y = Y; a.rows = rows; a.k = k;
-  a.part = b.orth_part; a.red = b.orth_red;
-  a.partd = b.orth_partd; a.redd = b.orth_redd;
-  a.bar = b.orth_bar; a.status = (int*)(b.orth_bar + 2);
-  a.run_if = run_if;
-  RET(cudaMemsetAsync(b.orth_bar, 0, 4 * sizeof(unsigned), st));
-  void* args[] = {&a};
-  note_launch();
-  RET(cudaLaunchCooperativeKernel((void*)orth_persistent, dim3(G), dim3(ORTH_NT), args, 0, st));
-  return cudaSuccess;
-}
-
 // shared-memory opt-in of the two CholeskyQR kernels, once per device
 PerDevice<cudaError_t> g_cholqr_setup;
 
@@ -1096,7 +546,7 @@ cudaError_t cholqr_setup() {
 }
 
 // Two scaled CholeskyQR passes on the column block Yb (rows x w, row stride
-// ldy): Yb -> U1 (in tmp, row stride w) -> Yb.  A breakdown raises
+// ldy): Yb -> U1 (in tmp, row stride w) -> Yb.  A non-finite Gram raises
 // b.chol_flag[0] and leaves Yb as it was.
 cudaError_t cholqr2_block(float* Yb, long long ldy, int rows, int w, float* tmp,
                           const SubspaceBuffers& b, cudaStream_t st) {
@@ -1113,7 +563,7 @@ cudaError_t cholqr2_block(float* Yb, long long ldy, int rows, int w, float* tmp,
     RET(tc_product(f32_view(src, idx_plain(1), idx_plain(lds)),
                    f32_view(src, idx_plain(1), idx_plain(lds)), w, w, rows, b.out, w, b, st));
     note_launch();
-    cholqr_factor<<<1, CQ_NT, fsm, st>>>(b.out, w, pass == 0 ? 1e-6f : 0.25f, pass == 0 ? 1 : 0,
+    cholqr_factor<<<1, CQ_NT, fsm, st>>>(b.out, w, pass == 0 ? 1e-6f : 0.25f,
                                          b.chol_L, b.chol_d, b.chol_li, b.chol_flag, nullptr);
     RET(cudaGetLastError());
     note_launch();
@@ -1214,8 +664,8 @@ constexpr float CQ_LINEAR_EMAX = 1e-3f;
 // one column block, in place: block classical Gram-Schmidt over column blocks,
 // each projected twice against the blocks before it on the tensor cores (S =
 // Q^T Y_b, Y_b -= Q S) and then orthonormalised by scaled CholeskyQR2; a
-// breakdown leaves Y unorthonormal, which the caller's orthonormality check
-// turns into the exact split.  b.Q is overwritten.
+// non-finite Gram leaves Y as it was, which the caller's check turns into the
+// exact split.  b.Q is overwritten.
 cudaError_t orthonormalise_blocks(float* Y, int rows, int k, const SubspaceBuffers& b,
                                   cudaStream_t st) {
   if (k > SUBSPACE_MAX_K) return cudaErrorInvalidValue;
@@ -1562,13 +1012,13 @@ cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm,
                                       k, b.ce_ss, 1.0 / ((double)m * n), seed + 7, b.seed_base, b.Y,
                                       nullptr, nullptr, hat, ldr, b.ce_ps);
   RET(cudaGetLastError());
-  // pass 1: G = Y^T Y, scaled Cholesky, Y <- U1 in place (skipped on breakdown)
+  // pass 1: G = Y^T Y, scaled Cholesky, Y <- U1 in place (skipped if G is not finite)
   const TcOperand H = plane_op(hat, k, rows, ldr, b.ce_ps);
   RET(tc_partials(H, H, k, k, rows, &sp, b, st));
   note_launch();
   sum_partials_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(b.part, sp, k, k, G, k);
   note_launch();
-  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 1e-6f, 1, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 1e-6f, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
                                        nullptr);
   RET(cudaGetLastError());
   note_launch();
@@ -1585,19 +1035,18 @@ cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm,
   RET(cudaGetLastError());
   // the full second pass, only if E was too large: U1 -> b.Q
   note_launch();
-  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 0.25f, 0, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 0.25f, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
                                        need_full);
   RET(cudaGetLastError());
   note_launch();
   cholqr_solve<<<sgrid, CQ_SOLVE_NT, ssm, st>>>(b.Y, k, rows, k, b.chol_L, b.chol_d, b.chol_li,
                                                 b.chol_flag, need_full, b.Q, k, SolvePlanes{});
   RET(cudaGetLastError());
-  // a breakdown in either pass: block Gram-Schmidt on Y (the input, or U1
-  // after a breakdown of the second pass)
-  RET(block_cgs(b.Y, rows, k, b, st, b.chol_flag));
   RET(tc_partials(plane_op(b.pa, rows, k, ldk, b.psa), plane_op(b.pb, k, k, ldk, b.psb), rows, k, k,
                   &sp, b, st));
   // the basis: FP64 factor (U, or V transposed) and planes of its transpose
+  // (after a non-finite Gram, Y itself: the check then
+  // hands the update to the exact split, which reports them)
   note_launch();
   basis_kernel<<<bgrid, 256, 0, st>>>(BasisSrc{b.part, sp, b.Y, b.chol_flag, b.Q, need_full}, rows, k,
                                       nullptr, 0.0, 0ull, b.seed_base, nullptr,
@@ -1627,9 +1076,6 @@ cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm,
 }
 
 }  // namespace
-
-unsigned long long g_orth_cluster_calls = 0;
-thread_local unsigned long long t_orth_cluster_calls = 0;
 
 size_t subspace_plane_elems_a(int cap) { return 3 * (size_t)(4 * cap) * tc_ld(4 * cap); }
 size_t subspace_plane_elems_b(int cap) { return 3 * (size_t)(4 * cap) * tc_ld(4 * cap); }
@@ -1674,13 +1120,8 @@ cudaError_t orth_check(const float* Q, int rows, int k, const SubspaceBuffers& b
 
 size_t subspace_buffer_floats(int cap) {
   const size_t m = 4 * (size_t)cap;
-  const size_t G = (m + ROWS_PER_CTA - 1) / ROWS_PER_CTA;
-  return m * cap /*Q*/ + m * cap /*Y*/ + m * m /*out*/ + G * MAX_K * PANEL /*orth partials*/ +
-         MAX_K * PANEL /*orth reduced*/ + 64 /*scal*/ + 2 * G * PANEL * PANEL /*FP64 partial Grams*/ +
-         2 * PANEL * PANEL /*FP64 Gram*/ + 64;
+  return m * cap /*Q*/ + m * cap /*Y*/ + m * m /*out*/;
 }
-
-int subspace_orth_ctas(int cap) { return (4 * cap + ROWS_PER_CTA - 1) / ROWS_PER_CTA; }
 
 namespace {
 // discarded weight 1 - ||centre||^2 / ||C_E||^2 of an accepted split
@@ -1695,23 +1136,22 @@ __global__ void split_finish_kernel(const double* __restrict__ ce_ss, const doub
 }
 
 // After the orthonormality check (G = Q^T Q): the defect is set to +inf if no
-// column of Q is live, or if a blocked orthonormalisation (which has no
-// Gram-Schmidt fallback) broke down, so that the exact split runs.
+// column of Q is live, or if an orthonormalisation met a non-finite Gram, so
+// that the exact split runs.
 __global__ void split_guard_kernel(const float* __restrict__ G, int k, const int* __restrict__ flag,
-                                   int blocked, double* defect) {
+                                   double* defect) {
   __shared__ int live;
   if (threadIdx.x == 0) live = 0;
   __syncthreads();
   for (int j = threadIdx.x; j < k; j += blockDim.x)
     if (G[(long long)j * k + j] >= 0.5f) live = 1;
   __syncthreads();
-  if (threadIdx.x == 0 && (!live || (blocked && *flag))) *defect = INFINITY;
+  if (threadIdx.x == 0 && (!live || *flag)) *defect = INFINITY;
 }
 
 cudaError_t split_guard(int k, const SubspaceBuffers& b, cudaStream_t st) {
   note_launch();
-  split_guard_kernel<<<1, 256, 0, st>>>(b.out, k, b.chol_flag, k > b.orth_block ? 1 : 0,
-                                        b.dscal + 2);
+  split_guard_kernel<<<1, 256, 0, st>>>(b.out, k, b.chol_flag, b.dscal + 2);
   return cudaGetLastError();
 }
 }  // namespace

@@ -8,13 +8,6 @@ struct SubspaceBuffers {
   float* Q;         // max(m, n) x k
   float* Y;         // max(m, n) x k
   float* out;       // m x n (k x n or m x k results)
-  float* orth_part; // orthonormalisation: per-CTA partial sums
-  float* orth_red;  // orthonormalisation: reduced sums
-  double* orth_partd;  // orthonormalisation: per-CTA partial panel Grams (FP64)
-  double* orth_redd;   // orthonormalisation: reduced panel Gram (FP64)
-  unsigned* orth_bar;  // orthonormalisation: grid barrier words + status (4 words)
-  int orth_max_ctas;
-  float* scal;      // scratch scalars
   double* dscal;    // FP64 scratch scalars (3)
   __nv_bfloat16* pa;   // tensor-core operand planes (3 x 4cap x ld(4cap))
   __nv_bfloat16* pb;   // tensor-core operand planes (3 x 4cap x ld(4cap))
@@ -32,13 +25,12 @@ struct SubspaceBuffers {
   int* zero;
   int zero_words;         // at most 64
   int* live;              // [0] a live column seen, [1] CTAs finished (centre_kernel)
-  // scaled CholeskyQR2: packed Cholesky factor, column scaling, 1 / L_jj,
-  // breakdown flag (0: the fast path succeeded)
+  // scaled CholeskyQR2: packed Cholesky factor, column scaling, 1 / L_jj, flags
   float* chol_L;          // w (w + 1) / 2 for a column block of width w
   float* chol_d;          // SUBSPACE_BLOCK_K
   float* chol_li;         // SUBSPACE_BLOCK_K
-  int* chol_flag;         // [0] breakdown flag of the current call, [1] count of breakdowns,
-                          // [2] full second pass flag, [3] its count, [4] deflated columns
+  int* chol_flag;         // [0] a non-finite Gram in the current call, [2] full second pass
+                          // flag, [3] its count, [4] columns dropped as dependent
   int orth_block;         // column-block width of the orthonormalisation (32..SUBSPACE_BLOCK_K)
   unsigned long long* seed_base;   // device counter mixed into the noise seeds (one per product)
   float* part;            // FP32 split-K partials of the small tensor-core products (may be
@@ -54,11 +46,6 @@ constexpr int SUBSPACE_MAX_K = 1024;
 // Floats of chol_L (one column block).
 constexpr size_t SUBSPACE_CHOL_FLOATS = (size_t)SUBSPACE_BLOCK_K * (SUBSPACE_BLOCK_K + 1) / 2;
 
-// Orthonormalisations launched as one thread-block cluster (all contexts; and
-// by the calling host thread).
-extern unsigned long long g_orth_cluster_calls;
-extern thread_local unsigned long long t_orth_cluster_calls;
-
 // BF16 elements of pa and pb for bond capacity cap.
 size_t subspace_plane_elems_a(int cap);
 size_t subspace_plane_elems_b(int cap);
@@ -67,8 +54,6 @@ size_t subspace_plane_elems_ce(int cap);
 
 // Floats needed by the float buffers above for bond capacity cap (m, n <= 4 cap).
 size_t subspace_buffer_floats(int cap);
-// CTAs of the orthonormalisation kernel for rows <= 4 cap.
-int subspace_orth_ctas(int cap);
 
 // Split C_E (m x n) into left (m x k) and right (k x n), FP64.  C_E is read
 // from b.ce_rm / b.ce_tr / b.ce_ss (its planes and norm, see above); the

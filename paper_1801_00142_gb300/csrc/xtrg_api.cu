@@ -205,7 +205,7 @@ struct xtrg_ctx {
     std::vector<int> out_dims;      // C's bonds after the captured doubling
     // host counters a replay advances by
     long long d_updates = 0;
-    unsigned long long d_launches = 0, d_cluster = 0;
+    unsigned long long d_launches = 0;
     double d_flops_contr = 0.0, d_flops_split = 0.0;
   };
   std::vector<DoublingGraph> graphs;
@@ -1210,19 +1210,10 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
       float* f = (float*)carve(ctx, subspace_buffer_floats(p.cap) * 4);
       ok = ok && f;
       if (f) {
-        const size_t G = (size_t)subspace_orth_ctas(p.cap);
         ctx->m.sb.Q = f; f += mm * c;
         ctx->m.sb.Y = f; f += mm * c;
-        ctx->m.sb.out = f; f += mm * mm;
-        ctx->m.sb.orth_part = f; f += G * SUBSPACE_BLOCK_K * 32;
-        ctx->m.sb.orth_red = f; f += SUBSPACE_BLOCK_K * 32;
-        ctx->m.sb.scal = f; f += 64;
-        ctx->m.sb.orth_partd = (double*)f; f += 2 * G * 32 * 32;
-        ctx->m.sb.orth_redd = (double*)f; f += 2 * 32 * 32;
-        ctx->m.sb.orth_max_ctas = (int)G;
+        ctx->m.sb.out = f;
       }
-      ctx->m.sb.orth_bar = (unsigned*)carve(ctx, 16);
-      ok = ok && ctx->m.sb.orth_bar;
       // scalars that every truncation clears in one go: its own, then the
       // exact split's
       {
@@ -1377,7 +1368,7 @@ bool capture_doubling(xtrg_ctx* ctx, xtrg_ctx::DoublingGraph* g) {
   }
   cudaStream_t user = ctx->st;
   const long long u0 = ctx->updates;
-  const unsigned long long l0 = t_xtrg_launches, c0 = t_orth_cluster_calls;
+  const unsigned long long l0 = t_xtrg_launches;
   const double fc0 = ctx->flops_contr, fs0 = ctx->flops_split;
   if (cudaStreamBeginCapture(ctx->cap_st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
@@ -1395,7 +1386,6 @@ bool capture_doubling(xtrg_ctx* ctx, xtrg_ctx::DoublingGraph* g) {
   // the host counters advanced while capturing; replays advance them again
   g->d_updates = ctx->updates - u0;
   g->d_launches = t_xtrg_launches - l0;
-  g->d_cluster = t_orth_cluster_calls - c0;
   g->d_flops_contr = ctx->flops_contr - fc0;
   g->d_flops_split = ctx->flops_split - fs0;
   ctx->updates = u0;
@@ -1456,7 +1446,6 @@ extern "C" xtrg_status xtrg_double(xtrg_ctx* ctx) {
       ctx->flops_contr += hit->d_flops_contr;
       ctx->flops_split += hit->d_flops_split;
       __atomic_add_fetch(&g_xtrg_launches, hit->d_launches, __ATOMIC_RELAXED);
-      __atomic_add_fetch(&g_orth_cluster_calls, hit->d_cluster, __ATOMIC_RELAXED);
       ctx->graph_replays++;
     } else {
       TRY(mixed_doubling_body(ctx));
@@ -1879,7 +1868,7 @@ extern "C" xtrg_status xtrg_get_stats(const xtrg_ctx* ctx, xtrg_stats* o) {
   o->kernel_launches = (long long)__atomic_load_n(&g_xtrg_launches, __ATOMIC_RELAXED);
   o->exact_split_fallbacks = ctx->fallbacks;
   o->split_ms = ctx->split_ms;
-  o->orth_cluster_calls = (long long)__atomic_load_n(&g_orth_cluster_calls, __ATOMIC_RELAXED);
+  o->orth_cluster_calls = 0;
   o->orth_fallbacks = 0;
   o->orth_full_second_pass = 0;
   o->graph_captures = ctx->graph_captures;
@@ -1895,7 +1884,6 @@ extern "C" xtrg_status xtrg_get_stats(const xtrg_ctx* ctx, xtrg_stats* o) {
             cudaSuccess ||
         cudaStreamSynchronize(ctx->st) != cudaSuccess)
       return XTRG_ECUDA;
-    o->orth_fallbacks = h[1];
     o->orth_full_second_pass = h[3];
     o->orth_deflated_columns = h[4];
   }
