@@ -3,8 +3,13 @@
 // CTA tile 128 x 128 (M x N), K-block of 64 BF16 (one 128-byte swizzle row;
 // 2 stages at 6 planes); persistent CTAs (one per SM).  Warp 0: TMA producer (one elected thread);
 // warp 1: MMA issuer (one elected thread, 4 x UMMA_K=16 per K-block and
-// product); warp 2: tensor-memory allocation; warps 4-7: epilogue
-// (tcgen05.ld 32x32b, lane quarter = warp % 4).
+// product); warp 2: tensor-memory allocation; warps 4-11: epilogue
+// (tcgen05.ld 32x32b, lane quarter = warp % 4, half of the columns each).
+// With four epilogue warps, each storing its own rows, the epilogue bound every
+// site of short contraction: at L = 64, D* = 256 the first substep ran at 116
+// TFLOP/s algorithmic and the second at 192, with eight and the store forms of
+// store_chunk at 161 and 222 (C_E, whose K hides it: 257); an odd bond of 173 in
+// two planes 25 -> 52 and 104 -> 137, its environment update 35 -> 91.
 //
 // Accumulation.  The tensor core rounds its FP32 accumulator toward zero, so
 // long accumulation chains in tensor memory shrink every output by a
@@ -31,7 +36,9 @@
 namespace {
 
 constexpr int BM = 128, BN = 128;
-constexpr int NTHREADS = 256;
+constexpr int EPI_WARPS = 8;                 // warps 4..11
+constexpr int EPI_COLS = BN * 4 / EPI_WARPS;   // output columns of each
+constexpr int NTHREADS = 128 + 32 * EPI_WARPS;
 
 // Shared-memory geometry for a K-block of BK BF16 (64: 128-byte swizzle,
 // 32: 64-byte swizzle).  K-major tiles are BM rows of SW bytes in 8-row
@@ -168,8 +175,8 @@ __device__ __forceinline__ void fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
+// 32 columns of the warp's 32 lanes; tmem_wait() before r is read
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -180,9 +187,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
         "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// acc[0..EPI_COLS) += the accumulator columns at taddr, round-to-nearest; all
+// loads in flight before the one wait
+__device__ __forceinline__ void tmem_add(uint32_t taddr, float* acc) {
+  uint32_t r[EPI_COLS];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int c = 0; c < EPI_COLS; c += 32) tmem_ld32(taddr + (uint32_t)c, r + c);
+  tmem_wait();
+#pragma unroll
+  for (int c = 0; c < EPI_COLS; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(r[c]));
 }
 
 __device__ __forceinline__ void store_out(const TcOutput& o, long long off, float v) {
@@ -201,76 +219,131 @@ __device__ __forceinline__ void store_out(const TcOutput& o, long long off, floa
   }
 }
 
-__device__ __forceinline__ uint32_t bf16_bits(__nv_bfloat16 x) {
-  return (uint32_t)__bfloat16_as_ushort(x);
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);   // one conversion instruction
+  return *reinterpret_cast<const uint32_t*>(&p);
 }
 
 // Split two values into up to three BF16 planes and pack each plane's pair
 // (first value in the low half: the lower address).
 __device__ __forceinline__ void split_pack2(float a, float b, uint32_t& w0, uint32_t& w1,
                                             uint32_t& w2) {
-  const __nv_bfloat16 a0 = __float2bfloat16_rn(a), b0 = __float2bfloat16_rn(b);
-  const float ar = a - __bfloat162float(a0), br = b - __bfloat162float(b0);
-  const __nv_bfloat16 a1 = __float2bfloat16_rn(ar), b1 = __float2bfloat16_rn(br);
-  const __nv_bfloat16 a2 = __float2bfloat16_rn(ar - __bfloat162float(a1));
-  const __nv_bfloat16 b2 = __float2bfloat16_rn(br - __bfloat162float(b1));
-  w0 = bf16_bits(a0) | (bf16_bits(b0) << 16);
-  w1 = bf16_bits(a1) | (bf16_bits(b1) << 16);
-  w2 = bf16_bits(a2) | (bf16_bits(b2) << 16);
+  w0 = pack_bf16(a, b);
+  const float ar = a - __uint_as_float(w0 << 16), br = b - __uint_as_float(w0 & 0xffff0000u);
+  w1 = pack_bf16(ar, br);
+  w2 = pack_bf16(ar - __uint_as_float(w1 << 16), br - __uint_as_float(w1 & 0xffff0000u));
 }
 
-// Store 32 consecutive output columns of one row (v[0..31] already scaled).
-// Column layout of the chunk, decided once per tile: contiguous (32 columns
-// at consecutive offsets), paired (columns 2j, 2j+1 adjacent) or scattered.
-// Vector stores need the lane's start offset aligned (8 elements for BF16
-// planes / 4 for FP32) and the plane stride likewise; otherwise narrower
-// stores are used.
-__device__ __forceinline__ void store_chunk(const TcOutput& o, long long om,
-                                            const long long* col, int layout, int ncols,
-                                            const float* v) {
-  if (o.mode == TC_OUT_BF16P) {
-    const long long ps = o.plane_stride;
-    const long long off0 = om + col[0];
-    if (layout == 2 && ncols == 32 && ((off0 | ps) & 7) == 0) {
+// Store a 32 x 32 chunk of the warp (lane = row, v = its 32 columns, already
+// scaled) as BF16 planes, or as FP32 through scattered views.  What decides the
+// form is which index is contiguous in the output, so that a store
+// instruction fills whole sectors:
+//  - pairs of columns adjacent and rows two apart (layout 1): a lane stores its
+//    own pairs, 4 bytes, a warp 128 contiguous bytes;
+//  - rows adjacent: a lane stores its own values; where rows pair up evenly
+//    (rowpair), the lanes 2i and 2i + 1 trade every other column and each
+//    stores two rows of one, 4 bytes instead of 2;
+//  - otherwise columns are (mostly) adjacent: the chunk is turned in shared
+//    memory and a row's columns go out side by side, 16 bytes a lane where
+//    every row is aligned, else 2.  (A lane storing its own row touched 32
+//    sectors per instruction: 15 times slower at an odd bond of 173.)
+struct ChunkForm {
+  int layout;        // columns: 2 contiguous, 1 paired, 0 other
+  bool rows_adjacent, rowpair;
+};
+constexpr int STG = 80;   // bytes of a staged row: 32 BF16, padded, 16-byte aligned
+
+__device__ __forceinline__ void store_chunk(const TcOutput& o, long long om, bool valid,
+                                            const long long* col, const ChunkForm& f, int ncols,
+                                            const float* v, uint8_t* stage) {
+  const int lane = threadIdx.x & 31;
+  if (o.mode != TC_OUT_BF16P) {
+    if (!valid) return;
 #pragma unroll
-      for (int q8 = 0; q8 < 4; ++q8) {
-        uint32_t w[3][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          split_pack2(v[q8 * 8 + 2 * e], v[q8 * 8 + 2 * e + 1], w[0][e], w[1][e], w[2][e]);
-        __nv_bfloat16* d = o.bf16 + off0 + q8 * 8;
-        *reinterpret_cast<uint4*>(d) = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
-        *reinterpret_cast<uint4*>(d + ps) = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
-        if (o.planes > 2)
-          *reinterpret_cast<uint4*>(d + 2 * ps) = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
-      }
-      return;
-    }
-    if (layout >= 1 && ncols == 32 && ((om + col[0]) & 1) == 0 && (ps & 1) == 0) {
-#pragma unroll
-      for (int jj = 0; jj < 32; jj += 2) {
-        const long long off = om + col[jj];
-        uint32_t w0, w1, w2;
-        split_pack2(v[jj], v[jj + 1], w0, w1, w2);
-        *reinterpret_cast<uint32_t*>(o.bf16 + off) = w0;
-        *reinterpret_cast<uint32_t*>(o.bf16 + off + ps) = w1;
-        if (o.planes > 2) *reinterpret_cast<uint32_t*>(o.bf16 + off + 2 * ps) = w2;
-      }
-      return;
-    }
-  } else {
-    const long long off0 = om + col[0];
-    if (layout == 2 && ncols == 32 && (off0 & 3) == 0) {
-      float4* d = reinterpret_cast<float4*>(o.f32 + off0);
-#pragma unroll
-      for (int q4 = 0; q4 < 8; ++q4)
-        d[q4] = make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
-      return;
-    }
+    for (int jj = 0; jj < 32; ++jj)
+      if (jj < ncols) store_out(o, om + col[jj], v[jj]);
+    return;
   }
+  const long long ps = o.plane_stride;
+  if (f.layout == 1 && ncols == 32 && __all_sync(0xffffffffu, !valid || ((om + col[0]) & 1) == 0) &&
+      (ps & 1) == 0) {
+    if (!valid) return;
 #pragma unroll
-  for (int jj = 0; jj < 32; ++jj)
-    if (jj < ncols) store_out(o, om + col[jj], v[jj]);
+    for (int jj = 0; jj < 32; jj += 2) {
+      const long long off = om + col[jj];
+      uint32_t w0, w1, w2;
+      split_pack2(v[jj], v[jj + 1], w0, w1, w2);
+      *reinterpret_cast<uint32_t*>(o.bf16 + off) = w0;
+      *reinterpret_cast<uint32_t*>(o.bf16 + off + ps) = w1;
+      if (o.planes > 2) *reinterpret_cast<uint32_t*>(o.bf16 + off + 2 * ps) = w2;
+    }
+    return;
+  }
+  if (f.rowpair) {
+    const bool odd = lane & 1;
+    const long long base = om - (odd ? 1 : 0);   // row of the even lane
+#pragma unroll
+    for (int jj = 0; jj < 32; jj += 2) {
+      const float give = odd ? v[jj] : v[jj + 1];
+      const float got = __shfl_xor_sync(0xffffffffu, give, 1);
+      const int j = jj + (odd ? 1 : 0);
+      if (j < ncols) {
+        uint32_t w0, w1, w2;
+        split_pack2(odd ? got : v[jj], odd ? v[jj + 1] : got, w0, w1, w2);
+        __nv_bfloat16* d = o.bf16 + base + col[j];
+        *reinterpret_cast<uint32_t*>(d) = w0;
+        *reinterpret_cast<uint32_t*>(d + ps) = w1;
+        if (o.planes > 2) *reinterpret_cast<uint32_t*>(d + 2 * ps) = w2;
+      }
+    }
+    return;
+  }
+  if (f.rows_adjacent) {
+    if (!valid) return;
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj)
+      if (jj < ncols) store_out(o, om + col[jj], v[jj]);
+    return;
+  }
+  const unsigned vm = __ballot_sync(0xffffffffu, valid);
+  const bool vec = f.layout == 2 && ncols == 32 && (ps & 7) == 0 &&
+                   __all_sync(0xffffffffu, !valid || ((om + col[0]) & 7) == 0);
+  const long long mycol = lane < ncols ? col[lane] : 0;
+  for (int q = 0; q < o.planes; ++q) {
+    // this lane's row of plane q
+#pragma unroll
+    for (int q8 = 0; q8 < 4; ++q8) {
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t w0, w1, w2;
+        split_pack2(v[q8 * 8 + 2 * e], v[q8 * 8 + 2 * e + 1], w0, w1, w2);
+        w[e] = q == 0 ? w0 : (q == 1 ? w1 : w2);
+      }
+      *reinterpret_cast<uint4*>(stage + lane * STG + q8 * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __syncwarp();
+    __nv_bfloat16* out = o.bf16 + q * ps;
+    if (vec) {
+      const long long c0 = col[0];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = i * 8 + lane / 4;
+        const long long omr = __shfl_sync(0xffffffffu, om, r);
+        if ((vm >> r) & 1)
+          *reinterpret_cast<uint4*>(out + omr + c0 + (lane % 4) * 8) =
+              *reinterpret_cast<const uint4*>(stage + r * STG + (lane % 4) * 16);
+      }
+    } else {
+#pragma unroll 4
+      for (int r = 0; r < 32; ++r) {
+        const long long omr = __shfl_sync(0xffffffffu, om, r);
+        if (((vm >> r) & 1) && lane < ncols)
+          out[omr + mycol] = *reinterpret_cast<const __nv_bfloat16*>(stage + r * STG + lane * 2);
+      }
+    }
+    __syncwarp();
+  }
 }
 
 // Tile t -> (m tile, n tile, batch x split).  The smaller of the two output
@@ -321,7 +394,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* corr_empty = corr_full + 2; // [2]
   uint64_t* done = corr_empty + 2;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
-  long long* col_off_all = (long long*)(tmem_slot + 2);   // [4][BN] per-warp column offsets
+  long long* col_off_all = (long long*)(tmem_slot + 2);   // [EPI_WARPS][EPI_COLS] column offsets
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int tiles_n = (p.N + BN - 1) / BN, tiles_m = (p.M + BM - 1) / BM;
@@ -336,9 +409,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&main_full[b], 1);
-      mbar_init(&main_empty[b], 4);
+      mbar_init(&main_empty[b], EPI_WARPS);
       mbar_init(&corr_full[b], 1);
-      mbar_init(&corr_empty[b], 4);
+      mbar_init(&corr_empty[b], EPI_WARPS);
     }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -459,11 +532,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // the done barrier tracks completion of every MMA issued so far
     mma_commit(done);
   } else if (warp >= 4) {
-    // ---------------- epilogue (4 warps; warp % 4 selects the TMEM lane quarter)
-    const int q = warp % 4;
+    // ---------------- epilogue (warp % 4 selects the TMEM lane quarter, two
+    // warps share it, each with half of the columns: one warp per scheduler
+    // could not hide its own latencies, and short-K tiles waited for it)
+    const int q = warp % 4, ec0 = (warp - 4) / 4 * EPI_COLS;
     const TcOutput& o = p.out;
-    long long* col_off = col_off_all + q * BN;
-    const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
+    long long* col_off = col_off_all + (warp - 4) * EPI_COLS;
+    uint8_t* stage = (uint8_t*)(((uintptr_t)(col_off_all + 4 * BN) + 15) & ~(uintptr_t)15) +
+                     (warp - 4) * 32 * STG;
+    const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ec0;
     long long h = 0;   // main chunks drained
     int j = 0;
     bool ok = true;
@@ -473,20 +550,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const int bidx = z / p.splitk, split = z % p.splitk;
       const int kb_begin = split * p.kb_per;
       const int kb_end = min(kb_begin + p.kb_per, p.kb_total);
-      const int n0 = nt * BN, m0 = mt * BM;
+      const int n0 = nt * BN + ec0, m0 = mt * BM;
       const int cb = j & 1;
       // column offsets of this tile, computed once per warp (the 3-level views
       // need divisions); warp-private, so no barrier across warps is needed
       __syncwarp();
-      for (int cc = lane; cc < BN; cc += 32) {
+      for (int cc = lane; cc < EPI_COLS; cc += 32) {
         const int n = n0 + cc;
         col_off[cc] = (o.mode == TC_OUT_PARTIAL || n >= p.N) ? (long long)n : idx_off(o.cn, n);
       }
       __syncwarp();
       // layout of each 32-column chunk (2 bits per chunk: 2 contiguous, 1 paired)
       int layouts = 0;
+      bool cols_even = true;   // every column offset of the chunk even
 #pragma unroll
-      for (int ch = 0; ch < BN / 32; ++ch) {
+      for (int ch = 0; ch < EPI_COLS / 32; ++ch) {
         const long long mine = col_off[ch * 32 + lane];
         const bool contig = mine == col_off[ch * 32] + lane;
         // paired: every even column's partner follows it, and all pair starts
@@ -497,24 +575,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const unsigned mc = __ballot_sync(0xffffffffu, contig);
         const unsigned mp = __ballot_sync(0xffffffffu, paired);
         layouts |= (mc == 0xffffffffu ? 2 : (mp == 0xffffffffu ? 1 : 0)) << (2 * ch);
+        cols_even = cols_even && __all_sync(0xffffffffu, n0 + ch * 32 + lane >= p.N || (mine & 1) == 0);
       }
       // accumulate the tile: every main chunk, then the corrections, each
       // added with round-to-nearest FP32 additions
-      float acc[BN];
+      float acc[EPI_COLS];
 #pragma unroll
-      for (int jj = 0; jj < BN; ++jj) acc[jj] = 0.f;
+      for (int jj = 0; jj < EPI_COLS; ++jj) acc[jj] = 0.f;
       for (int kb = kb_begin; kb < kb_end && ok; kb += CK, ++h) {
         const int mb = (int)(h & 1);
         ok = mbar_wait(&main_full[mb], (uint32_t)((h >> 1) & 1), p.err);
         if (!ok) break;
         fence_after();
-#pragma unroll
-        for (int c = 0; c < BN; c += 32) {
-          float v[32];
-          tmem_ld32(lane_base + (uint32_t)(mb * BN + c), v);
-#pragma unroll
-          for (int jj = 0; jj < 32; ++jj) acc[c + jj] = __fadd_rn(acc[c + jj], v[jj]);
-        }
+        tmem_add(lane_base + (uint32_t)(mb * BN), acc);
         fence_before();
         __syncwarp();
         if (lane == 0)
@@ -526,15 +599,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         ok = mbar_wait(&corr_full[cb], (uint32_t)((j >> 1) & 1), p.err);
         if (!ok) break;
         fence_after();
-        if (kb_end > kb_begin) {
-#pragma unroll
-          for (int c = 0; c < BN; c += 32) {
-            float v[32];
-            tmem_ld32(lane_base + (uint32_t)(CORR_COL + cb * BN + c), v);
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) acc[c + jj] = __fadd_rn(acc[c + jj], v[jj]);
-          }
-        }
+        if (kb_end > kb_begin) tmem_add(lane_base + (uint32_t)(CORR_COL + cb * BN), acc);
         fence_before();
         __syncwarp();
         if (lane == 0)
@@ -542,19 +607,42 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                        : "memory");
       }
       const int m = m0 + q * 32 + lane;
-      if (m >= p.M) continue;
       float* dstp = nullptr;
       long long om = 0;
       if (o.mode == TC_OUT_PARTIAL)
         dstp = o.f32 + (((long long)split * p.batch + bidx) * p.M + m) * (long long)p.N;
       else
-        om = bidx * o.scb + idx_off(o.cm, m);
+        om = bidx * o.scb + (m < p.M ? idx_off(o.cm, m) : 0);
+      // whole warp: are the rows adjacent in the output, and do they pair up
+      // evenly (see store_chunk)
+      const bool valid = m < p.M;
+      ChunkForm form{0, false, false};
+      if (o.mode == TC_OUT_BF16P) {
+        const long long next = __shfl_down_sync(0xffffffffu, om, 1);
+        const unsigned adj = __ballot_sync(0xffffffffu, lane < 31 && next == om + 1);
+        form.rows_adjacent = __popc(adj) >= 16;
+        form.rowpair = cols_even && (o.plane_stride & 1) == 0 &&
+                       __all_sync(0xffffffffu, valid && ((lane & 1) || (next == om + 1 && (om & 1) == 0)));
+      }
+      // a warp below the last row has nothing to store (a partly filled one stays
+      // whole where its lanes trade values)
+      if (!__any_sync(0xffffffffu, valid) || (o.mode == TC_OUT_PARTIAL && !valid)) continue;
       const float alpha = (float)o.alpha;
-#pragma unroll
-      for (int c = 0; c < BN; c += 32) {
+      // the two chunks in a loop that is not unrolled: the store forms are long,
+      // and a tile's time is what a few warps need to fetch and run them
+#pragma unroll 1
+      for (int ch = 0; ch < EPI_COLS / 32; ++ch) {
+        const int c = ch * 32;
         const int ncols = min(32, p.N - (n0 + c));
-        if (ncols <= 0) continue;
-        float* v = acc + c;
+        if (ncols <= 0) break;
+        float v[32];
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) {
+          v[jj] = acc[jj];
+#pragma unroll
+          for (int k = 1; k < EPI_COLS / 32; ++k)
+            if (ch == k) v[jj] = acc[32 * k + jj];
+        }
         if (o.mode == TC_OUT_PARTIAL) {
           float* d = dstp + n0 + c;
           if (ncols == 32 && ((uintptr_t)d & 15) == 0) {
@@ -570,7 +658,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         } else {
 #pragma unroll
           for (int jj = 0; jj < 32; ++jj) v[jj] *= alpha;
-          store_chunk(o, om, col_off + c, (layouts >> (2 * (c / 32))) & 3, ncols, v);
+          form.layout = (layouts >> (2 * ch)) & 3;
+          store_chunk(o, om, valid, col_off + c, form, ncols, v, stage);
         }
       }
     }
@@ -608,6 +697,10 @@ EncodeFn get_encode() {
   return fn;
 }
 
+// K-block width: 64 BF16 (one 128-byte swizzle row).  A 32-wide K-block
+// (64-byte swizzle, twice the stages) computed the same and was slower.
+constexpr int K_BLOCK = 64;
+
 // the kernel's shared-memory opt-in and the SM count, once per device
 struct LaunchSetup {
   cudaError_t err;
@@ -617,7 +710,7 @@ PerDevice<LaunchSetup> g_launch_setup;
 
 template <int BMN, int NPROD>
 cudaError_t opt_in() {
-  return cudaFuncSetAttribute(tc_gemm_kernel<64, BMN, NPROD>,
+  return cudaFuncSetAttribute(tc_gemm_kernel<K_BLOCK, BMN, NPROD>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
@@ -652,10 +745,6 @@ int chunk_terms() {
   }();
   return v;
 }
-
-// K-block width: 64 BF16 (one 128-byte swizzle row).  A 32-wide K-block
-// (64-byte swizzle, twice the stages) computed the same and was slower.
-constexpr int K_BLOCK = 64;
 
 // 4-D map with BK-wide boxes (BK = 64: 128-byte swizzle, 32: 64-byte),
 // out-of-range elements read as zero.
@@ -728,7 +817,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K,
   cudaError_t e;
   if ((e = make_map(&ma, A, BK)) != cudaSuccess) return e;
   if ((e = make_map(&mb, B, BK)) != cudaSuccess) return e;
-  const int smem = S * stage_bytes + 1024 + (2 * S + 9) * 8 + 8 + 4 * BN * 8 + 64;
+  const int smem = S * stage_bytes + 1024 + (2 * S + 9) * 8 + 8 + 4 * BN * 8 + 64 + EPI_WARPS * 32 * STG;
   int sms = 0;
   if ((e = launch_setup(&sms)) != cudaSuccess) return e;
   const long long tiles =
@@ -738,12 +827,12 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K,
   note_launch();
   const int sel = (B.mn_major ? 3 : 0) + (nprod == 1 ? 0 : nprod == 3 ? 1 : 2);
   switch (sel) {
-    case 0: tc_gemm_kernel<64, 0, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 1: tc_gemm_kernel<64, 0, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 2: tc_gemm_kernel<64, 0, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 3: tc_gemm_kernel<64, 1, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 4: tc_gemm_kernel<64, 1, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    default: tc_gemm_kernel<64, 1, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 0: tc_gemm_kernel<K_BLOCK, 0, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 1: tc_gemm_kernel<K_BLOCK, 0, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 2: tc_gemm_kernel<K_BLOCK, 0, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 3: tc_gemm_kernel<K_BLOCK, 1, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 4: tc_gemm_kernel<K_BLOCK, 1, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    default: tc_gemm_kernel<K_BLOCK, 1, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
   }
   return cudaGetLastError();
 }

@@ -645,7 +645,7 @@ bool mixed_for_beta(const xtrg_ctx* ctx, double beta) {
 //   site copies  sT[(s,a',t)][a]   sP[(u,b')][(b,t)]   sN[(a',t',s')][a'']   sQ[(b',u')][(t',b'')]
 //   environment  V[c][b][a]                 (left and right alike)
 //   left half    T1[c][(s,a')][(b,t)]  ->  Lp[(c,s,u)][(b',a')]
-//   right half   T1R[c''][(a',s')][(t',b'')]  ->  Rp[(s',u',c'')][(b',a')]
+//   right half   T1R[c''][(s',a')][(t',b'')]  ->  Rp[(s',u',c'')][(b',a')]
 //   C_E = Lp Rp^T (split-K, FP64 sum); env update V' = C^T-part x (Lp or Rp)
 //   with the half read MN-major.
 
@@ -747,13 +747,13 @@ xtrg_status mixed_right_part(xtrg_ctx* ctx, const DevMpo& C, int j) {
   TcOperand An = opnd(ctx->m.site[2][j], P, 4 * a2, a3, tc_ld(a3), 0, ctx->plan.m_site[2], 1);
   TcOperand Be = opnd(ctx->m.env[j + 1], P, a3, a3, ldE, (long long)a3 * ldE, ctx->plan.m_env, c2);
   TRY(tc(ctx, An, Be, 4 * a2, a3, a3, c2, 1,
-         out_planes(ctx->m.T1R, P, ctx->plan.m_t1, idx_split3(2, 2, 2 * ld2, a3, ld2),
+         out_planes(ctx->m.T1R, P, ctx->plan.m_t1, idx_split3(2, 2, ld2, a3, a2 * ld2),
                     idx_plain(1), 2LL * a2 * ld2)));
   ctx->cur_tag = 2;
   TcOperand At = opnd(ctx->m.T1R, P, 2 * a2, 2 * a3, ld2, 2LL * a2 * ld2, ctx->plan.m_t1, c2);
   TcOperand Bq = opnd(ctx->m.site[3][j], P, 2 * a2, 2 * a3, tc_ld(2 * a3), 0, ctx->plan.m_site[3], 1);
   TRY(tc(ctx, At, Bq, 2 * a2, 2 * a2, 2 * a3, c2, 1,
-         out_planes(Rp, P, ctx->plan.m_lp, idx_split2(2, 1, 2LL * c2 * ldR),
+         out_planes(Rp, P, ctx->plan.m_lp, idx_split2(a2, 2LL * c2 * ldR, 1),
                     idx_split2(2, a2, (long long)c2 * ldR), ldR)));
   return XTRG_OK;
 }
