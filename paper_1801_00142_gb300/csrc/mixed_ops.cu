@@ -30,52 +30,69 @@ inline int grid_for(long long n) {
 // and FP64 conversions.
 constexpr int TP_R = 32, TP_K = 64;
 template <typename S>
+struct PlaneJob {
+  const S* src;
+  Idx3 rv, kv;
+  long long sbs;
+  int rows, K, tiles_r, tiles_k;
+  long long tiles;
+  __nv_bfloat16* out;
+  long long ld, obs, ops;
+  int kfast, vec;   // reads along k; 16-byte stores
+};
+
+// One matrix, or with PAIR two in one launch (a small product's operands);
+// clear (may be null) is set to zero.  With run_if, runs only if *run_if >
+// thresh or is not finite.
+template <typename S, bool PAIR>
 __global__ void __launch_bounds__(256)
-    to_planes_kernel(const S* __restrict__ src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
-                     int tiles_r, int tiles_k, long long tiles, __nv_bfloat16* __restrict__ out,
-                     long long ld, long long obs, int planes, long long ops, int kfast, int vec,
+    to_planes_kernel(const PlaneJob<S> j0, const PlaneJob<S> j1, int planes, int* clear,
                      const double* __restrict__ run_if, double thresh) {
   if (run_if && *run_if <= thresh) return;
   __shared__ __align__(16) unsigned short tp[3][TP_R][TP_K + 8];
   const int tid = threadIdx.x;
-  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int b = (int)(t / (tiles_r * tiles_k)), w = (int)(t - (long long)b * (tiles_r * tiles_k));
-    const int r0 = w / tiles_k * TP_R, k0 = w % tiles_k * TP_K;
-    const S* sb = src + b * sbs;
+  if (clear && blockIdx.x == 0 && tid == 0) *clear = 0;
+  for (long long tt = blockIdx.x; tt < j0.tiles + j1.tiles; tt += gridDim.x) {
+    const PlaneJob<S>& j = !PAIR || tt < j0.tiles ? j0 : j1;
+    const long long t = !PAIR || tt < j0.tiles ? tt : tt - j0.tiles;
+    const int per = j.tiles_r * j.tiles_k;
+    const int b = (int)(t / per), w = (int)(t - (long long)b * per);
+    const int r0 = w / j.tiles_k * TP_R, k0 = w % j.tiles_k * TP_K;
+    const S* sb = j.src + b * j.sbs;
     S x[8];
-    if (kfast) {
+    if (j.kfast) {
       const int k = k0 + tid % 64, y = tid / 64;
-      const long long ok = k < K ? off32(kv, k) : 0;
+      const long long ok = k < j.K ? off32(j.kv, k) : 0;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int r = r0 + y + 4 * u;
-        x[u] = (r < rows && k < K) ? sb[off32(rv, r) + ok] : S(0);
+        x[u] = (r < j.rows && k < j.K) ? sb[off32(j.rv, r) + ok] : S(0);
       }
     } else {
       const int r = r0 + tid % 32, y = tid / 32;
-      const long long orr = r < rows ? off32(rv, r) : 0;
+      const long long orr = r < j.rows ? off32(j.rv, r) : 0;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int k = k0 + y + 8 * u;
-        x[u] = (r < rows && k < K) ? sb[orr + off32(kv, k)] : S(0);
+        x[u] = (r < j.rows && k < j.K) ? sb[orr + off32(j.kv, k)] : S(0);
       }
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       unsigned short c[3];
       cut(x[u], c);
-      const int y = kfast ? tid / 64 + 4 * u : tid % 32;
-      const int z = kfast ? tid % 64 : tid / 32 + 8 * u;
+      const int y = j.kfast ? tid / 64 + 4 * u : tid % 32;
+      const int z = j.kfast ? tid % 64 : tid / 32 + 8 * u;
       tp[0][y][z] = c[0];
       tp[1][y][z] = c[1];
       tp[2][y][z] = c[2];
     }
     __syncthreads();
     const int y = tid / 8, z = tid % 8 * 8, r = r0 + y, k = k0 + z;
-    if (r < rows && k < ld) {
-      __nv_bfloat16* d = out + b * obs + (long long)r * ld + k;
-      for (int q = 0; q < planes; ++q, d += ops) {
-        if (vec) {
+    if (r < j.rows && k < j.ld) {
+      __nv_bfloat16* d = j.out + b * j.obs + (long long)r * j.ld + k;
+      for (int q = 0; q < planes; ++q, d += j.ops) {
+        if (j.vec) {
           *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(&tp[q][y][z]);
         } else {
           for (int u = 0; u < 8; ++u) d[u] = __ushort_as_bfloat16(tp[q][y][z + u]);
@@ -94,34 +111,53 @@ int unit_stride(const Idx3& d) {
 }
 
 template <typename S>
-cudaError_t launch_to_planes(const S* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
-                             int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
-                             long long ops, cudaStream_t st, const double* run_if = nullptr,
-                             double thresh = 0.0) {
-  if ((long long)rows * ld * batch <= 0) return cudaSuccess;
-  const int tiles_r = (rows + TP_R - 1) / TP_R, tiles_k = (int)((ld + TP_K - 1) / TP_K);
-  const long long tiles = (long long)tiles_r * tiles_k * batch;
-  const int vec = ((uintptr_t)out % 16) == 0 && ld % 8 == 0 && obs % 8 == 0 && ops % 8 == 0;
-  const int kfast = unit_stride(kv) || !unit_stride(rv);
-  const long long grid = tiles < 152 * 16 ? tiles : 152 * 16;
+PlaneJob<S> plane_job(const S* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K, int batch,
+                      __nv_bfloat16* out, long long ld, long long obs, long long ops) {
+  PlaneJob<S> j{};
+  if ((long long)rows * ld * batch <= 0) return j;
+  j.src = src; j.rv = rv; j.kv = kv; j.sbs = sbs; j.rows = rows; j.K = K;
+  j.tiles_r = (rows + TP_R - 1) / TP_R;
+  j.tiles_k = (int)((ld + TP_K - 1) / TP_K);
+  j.tiles = (long long)j.tiles_r * j.tiles_k * batch;
+  j.out = out; j.ld = ld; j.obs = obs; j.ops = ops;
+  j.vec = ((uintptr_t)out % 16) == 0 && ld % 8 == 0 && obs % 8 == 0 && ops % 8 == 0;
+  j.kfast = unit_stride(kv) || !unit_stride(rv);
+  return j;
+}
+
+template <typename S>
+cudaError_t launch_to_planes(const PlaneJob<S>& j0, const PlaneJob<S>& j1, int planes, int* clear,
+                             cudaStream_t st, const double* run_if = nullptr, double thresh = 0.0) {
+  const long long tiles = j0.tiles + j1.tiles;
+  if (tiles <= 0) return cudaSuccess;
+  // two matrices share a launch while they leave room on the chip; larger ones
+  // gain nothing by it, and the kernel of one has its view in constants (1024 x
+  // 65536: 157 us a matrix, 180 us in a pair)
+  if (j0.tiles > 0 && j1.tiles > 0 && tiles > 152 * 16) {
+    const cudaError_t e = launch_to_planes(j0, PlaneJob<S>{}, planes, clear, st, run_if, thresh);
+    return e != cudaSuccess ? e : launch_to_planes(j1, PlaneJob<S>{}, planes, nullptr, st, run_if, thresh);
+  }
+  const unsigned grid = (unsigned)(tiles < 152 * 16 ? tiles : 152 * 16);
   note_launch();
-  to_planes_kernel<S><<<(unsigned)grid, 256, 0, st>>>(src, rv, kv, sbs, rows, K, tiles_r, tiles_k,
-                                                      tiles, out, ld, obs, planes, ops, kfast, vec, run_if,
-                                                      thresh);
+  if (j1.tiles == 0)
+    to_planes_kernel<S, false><<<grid, 256, 0, st>>>(j0, j1, planes, clear, run_if, thresh);
+  else
+    to_planes_kernel<S, true><<<grid, 256, 0, st>>>(j0, j1, planes, clear, run_if, thresh);
   return cudaGetLastError();
 }
 
+// FP64 sum of FP32 partials; the conversions are integer operations (FP64-pipe
+// conversions alone bound this kernel: 13 us on 2.7 M elements)
 __global__ void reduce_partials_kernel(const float* __restrict__ part, int splits, long long n,
                                        double* __restrict__ out) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
-    double s = 0.0;
+    double s = f32_to_f64(part[e]);
 #pragma unroll 8
-    for (int i = 0; i < splits; ++i) s += (double)part[i * n + e];
+    for (int i = 1; i < splits; ++i) s += f32_to_f64(part[i * n + e]);
     out[e] = s;
   }
 }
-
 
 // One 32 x 32 tile of C = sum of the split-K partials: the FP64 result, its
 // three BF16 planes in both orientations (row-major [m][ldn] and transposed
@@ -226,21 +262,35 @@ __global__ void reduce_partials_planes_kernel(const float* __restrict__ part, in
 cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                       int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                       long long ops, cudaStream_t st) {
-  return launch_to_planes<double>(src, rv, kv, sbs, rows, K, batch, out, ld, obs, planes, ops, st);
+  return launch_to_planes(plane_job(src, rv, kv, sbs, rows, K, batch, out, ld, obs, ops),
+                          PlaneJob<double>{}, planes, nullptr, st);
+}
+
+cudaError_t to_planes_pair(const double* a, int rows_a, int Ka, __nv_bfloat16* out_a, const double* b,
+                           int rows_b, int Kb, __nv_bfloat16* out_b, int batch, int planes,
+                           int* clear, cudaStream_t st) {
+  const long long lda = (Ka + 7) / 8 * 8, ldb = (Kb + 7) / 8 * 8;
+  return launch_to_planes(
+      plane_job(a, idx_plain(Ka), idx_plain(1), (long long)rows_a * Ka, rows_a, Ka, batch, out_a, lda,
+                rows_a * lda, batch * rows_a * lda),
+      plane_job(b, idx_plain(Kb), idx_plain(1), (long long)rows_b * Kb, rows_b, Kb, batch, out_b, ldb,
+                rows_b * ldb, batch * rows_b * ldb),
+      planes, clear, st);
 }
 
 cudaError_t to_planes_if(const double* src, Idx3 rv, Idx3 kv, int rows, int K, __nv_bfloat16* out,
                          long long ld, int planes, long long ops, const double* run_if,
                          double thresh, cudaStream_t st) {
   if (!run_if) return cudaErrorInvalidValue;
-  return launch_to_planes<double>(src, rv, kv, 0, rows, K, 1, out, ld, 0, planes, ops, st, run_if,
-                                  thresh);
+  return launch_to_planes(plane_job(src, rv, kv, 0, rows, K, 1, out, ld, 0, ops), PlaneJob<double>{},
+                          planes, nullptr, st, run_if, thresh);
 }
 
 cudaError_t to_planes_f32(const float* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                           int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                           long long ops, cudaStream_t st) {
-  return launch_to_planes<float>(src, rv, kv, sbs, rows, K, batch, out, ld, obs, planes, ops, st);
+  return launch_to_planes(plane_job(src, rv, kv, sbs, rows, K, batch, out, ld, obs, ops),
+                          PlaneJob<float>{}, planes, nullptr, st);
 }
 
 cudaError_t reduce_partials(const float* part, int splits, long long n, double* out,

@@ -45,6 +45,15 @@ __device__ __forceinline__ void cut(S x, unsigned short* w) {
   w[2] = __bfloat16_as_ushort(p2);
 }
 
+// an FP32 value as FP64, by integer operations for normal values
+__device__ __forceinline__ double f32_to_f64(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xff;
+  if (e - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u)),
+                            (int)(u << 29));
+  return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)x;
+}
+
 // offset of a view's index with 32-bit divisions (indices are below 2^31)
 __device__ __forceinline__ long long off32(const Idx3& d, unsigned idx) {
   if (d.n0 == 1 && d.n1 == 1) return (long long)idx * d.s2;

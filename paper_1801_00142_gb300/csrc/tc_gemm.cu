@@ -31,6 +31,7 @@
 #include <stdint.h>
 #include <stdlib.h>
 
+#include "planes.cuh"
 #include "tc_gemm.cuh"
 
 namespace {
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       __syncwarp();
       for (int cc = lane; cc < EPI_COLS; cc += 32) {
         const int n = n0 + cc;
-        col_off[cc] = (o.mode == TC_OUT_PARTIAL || n >= p.N) ? (long long)n : idx_off(o.cn, n);
+        col_off[cc] = (o.mode >= TC_OUT_PARTIAL || n >= p.N) ? (long long)n : idx_off(o.cn, n);
       }
       __syncwarp();
       // layout of each 32-column chunk (2 bits per chunk: 2 contiguous, 1 paired)
@@ -611,7 +612,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       long long om = 0;
       if (o.mode == TC_OUT_PARTIAL)
         dstp = o.f32 + (((long long)split * p.batch + bidx) * p.M + m) * (long long)p.N;
-      else
+      else if (o.mode != TC_OUT_F64)
         om = bidx * o.scb + (m < p.M ? idx_off(o.cm, m) : 0);
       // whole warp: are the rows adjacent in the output, and do they pair up
       // evenly (see store_chunk)
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       // a warp below the last row has nothing to store (a partly filled one stays
       // whole where its lanes trade values)
-      if (!__any_sync(0xffffffffu, valid) || (o.mode == TC_OUT_PARTIAL && !valid)) continue;
+      if (!__any_sync(0xffffffffu, valid) || (o.mode >= TC_OUT_PARTIAL && !valid)) continue;
       const float alpha = (float)o.alpha;
       // the two chunks in a loop that is not unrolled: the store forms are long,
       // and a tile's time is what a few warps need to fetch and run them
@@ -643,7 +644,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           for (int k = 1; k < EPI_COLS / 32; ++k)
             if (ch == k) v[jj] = acc[32 * k + jj];
         }
-        if (o.mode == TC_OUT_PARTIAL) {
+        if (o.mode == TC_OUT_F64) {
+          double* d = o.f64 + ((long long)bidx * p.M + m) * (long long)p.N + n0 + c;
+          if (ncols == 32 && ((uintptr_t)d & 15) == 0) {
+#pragma unroll
+            for (int q2 = 0; q2 < 16; ++q2)
+              reinterpret_cast<double2*>(d)[q2] =
+                  make_double2(f32_to_f64(v[2 * q2]), f32_to_f64(v[2 * q2 + 1]));
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 32; ++jj)
+              if (jj < ncols) d[jj] = f32_to_f64(v[jj]);
+          }
+        } else if (o.mode == TC_OUT_PARTIAL) {
           float* d = dstp + n0 + c;
           if (ncols == 32 && ((uintptr_t)d & 15) == 0) {
 #pragma unroll

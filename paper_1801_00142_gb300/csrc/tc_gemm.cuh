@@ -17,7 +17,8 @@
 enum TcOutMode {
   TC_OUT_F32 = 0,      // FP32 values scattered through (cm, cn, scb)
   TC_OUT_BF16P = 1,    // BF16 split planes scattered through (cm, cn, scb)
-  TC_OUT_PARTIAL = 2   // FP32 split-K partials, plain [split][batch][M][N]
+  TC_OUT_PARTIAL = 2,  // FP32 split-K partials, plain [split][batch][M][N]
+  TC_OUT_F64 = 3       // the FP32 result widened, plain [batch][M][N] (splitk = 1)
 };
 
 struct TcOperand {
@@ -35,6 +36,7 @@ struct TcOperand {
 struct TcOutput {
   int mode;
   float* f32;
+  double* f64;
   __nv_bfloat16* bf16;
   int planes;                  // BF16 planes written (2 or 3)
   long long plane_stride;

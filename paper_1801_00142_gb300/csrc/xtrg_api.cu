@@ -1938,6 +1938,25 @@ xtrg_status tc_gemm_check_args(const double* A, const double* B, double* C, int 
   return XTRG_OK;
 }
 
+namespace {
+// One pinned int per host thread (a call waits for its own copy before it
+// returns), given back when the thread ends; null if it cannot be had.
+int* pinned_flag() {
+  struct Pinned {
+    int* p = nullptr;
+    ~Pinned() {
+      if (p) cudaFreeHost(p);
+    }
+  };
+  static thread_local Pinned f;
+  if (!f.p && cudaHostAlloc((void**)&f.p, sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    f.p = nullptr;
+  }
+  return f.p;
+}
+}  // namespace
+
 xtrg_status tc_gemm_run(const double* A, const double* B, double* C, int M, int N, int K, int batch,
                         int planes, int nprod, int splitk, char* base, cudaStream_t st, bool b_kn) {
   const TcGemmScratch w = tc_gemm_scratch(M, N, K, batch, planes, splitk, b_kn);
@@ -1949,34 +1968,33 @@ xtrg_status tc_gemm_run(const double* A, const double* B, double* C, int M, int 
   const long long ldn = tc_ld(N);
   const long long psA = (long long)batch * M * ld;
   const long long psB = b_kn ? (long long)batch * K * ldn : (long long)batch * N * ld;
-  if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return XTRG_ECUDA;
-  if (to_planes(A, idx_plain(K), idx_plain(1), (long long)M * K, M, K, batch, pa, ld,
-                (long long)M * ld, planes, psA, st) != cudaSuccess)
+  // both operands' planes (B: its rows of K, K-major, or its own K x N rows,
+  // MN-major) and the cleared error flag in one launch
+  if ((b_kn ? to_planes_pair(A, M, K, pa, B, K, N, pb, batch, planes, err, st)
+            : to_planes_pair(A, M, K, pa, B, N, K, pb, batch, planes, err, st)) != cudaSuccess)
     return XTRG_ECUDA;
-  // B^T rows (K-major), or B's own K x N rows (MN-major operand)
-  const cudaError_t eb =
-      b_kn ? to_planes(B, idx_plain(N), idx_plain(1), (long long)K * N, K, N, batch, pb, ldn,
-                       (long long)K * ldn, planes, psB, st)
-           : to_planes(B, idx_plain(K), idx_plain(1), (long long)N * K, N, K, batch, pb, ld,
-                       (long long)N * ld, planes, psB, st);
-  if (eb != cudaSuccess) return XTRG_ECUDA;
   TcOperand oa{pa, planes, M, K, ld, (long long)M * ld, psA, batch};
   TcOperand ob{pb, planes, N, K, ld, (long long)N * ld, psB, batch};
   if (b_kn) ob = TcOperand{pb, planes, N, K, ldn, (long long)K * ldn, psB, batch, 1};
   TcOutput out;
   memset(&out, 0, sizeof out);
-  out.mode = TC_OUT_PARTIAL;
+  out.mode = splitk == 1 ? TC_OUT_F64 : TC_OUT_PARTIAL;
   out.f32 = part;
+  out.f64 = C;
   out.alpha = 1.0;
   if (tc_gemm(oa, ob, M, N, K, batch, nprod, splitk, out, err, st) != cudaSuccess)
     return XTRG_ECUDA;
-  if (reduce_partials(part, splitk, (long long)batch * M * N, C, st) != cudaSuccess)
+  if (splitk > 1 && reduce_partials(part, splitk, (long long)batch * M * N, C, st) != cudaSuccess)
     return XTRG_ECUDA;
-  int h = 0;
-  if (cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+  // the error flag comes back into pinned memory (a copy into pageable memory
+  // is staged and waits on the host a second time)
+  int pageable = 0;
+  int* h = pinned_flag();
+  if (!h) h = &pageable;
+  if (cudaMemcpyAsync(h, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return XTRG_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return XTRG_ECUDA;
-  return h ? XTRG_ETIMEOUT : XTRG_OK;
+  return *h ? XTRG_ETIMEOUT : XTRG_OK;
 }
 
 extern "C" size_t xtrg_tc_gemm_workspace_bytes(int M, int N, int K, int batch, int planes,
