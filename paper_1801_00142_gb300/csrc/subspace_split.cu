@@ -229,7 +229,8 @@ size_t cholqr_factor_smem(int k) {
 // 32-wide panels: the diagonal block in registers of warp 0 (lane = row, shuffles),
 // the rows below it one per thread against that block, then the trailing
 // update in 4 x 4 register blocks from the transposed panel copy (float4
-// reads, conflict-free).  With run_if set, runs only if *run_if != 0 and
+// reads, conflict-free).  Measured at k = 64: 34 us with a column at a time and
+// a row's loads at a time, 22 us so.  With run_if set, runs only if *run_if != 0 and
 // *flag == 0.
 __global__ void __launch_bounds__(CQ_NT, 1)
     cholqr_factor(const float* __restrict__ G, int k, float tau, float* __restrict__ Lout, float* __restrict__ dout, float* __restrict__ linv_out,
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(CQ_NT, 1)
   float* li = d + MAX_K;                            // 1 / L_jj
   __shared__ float red[32];
   __shared__ int bad, ndefl;
-  __shared__ __align__(16) float colb[32];   // column of the diagonal-block step
+  __shared__ float4 colb[32];   // four columns of the diagonal-block step
   const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
   float gm = 0.f;
   for (int j = tid; j < k; j += CQ_NT) {
@@ -271,24 +272,33 @@ __global__ void __launch_bounds__(CQ_NT, 1)
     d[j] = (g > 1e-30f * gmax && g < 3.0e38f) ? 1.f / sqrtf(g) : 0.f;
   }
   __syncthreads();
-  // packed load, row by row (one warp per row, coalesced reads of G); the
-  // row's eight loads are issued before any is used, so a warp waits on the
-  // memory latency once per row rather than once per 32 columns
-  for (int i = warp; i < k; i += CQ_NT / 32) {
-    const float di = d[i];
-    float g[MAX_K / 32];
+  // packed load, a warp per row (coalesced reads of G), three rows at a time:
+  // all their loads are issued before any is used, so a warp waits out the
+  // memory latency once per three rows
+  constexpr int LR = 3;
+  for (int i0 = warp; i0 < k; i0 += LR * (CQ_NT / 32)) {
+    float g[LR][MAX_K / 32];
 #pragma unroll
-    for (int t = 0; t < MAX_K / 32; ++t) {
-      const int j = lane + 32 * t;
-      g[t] = j <= i ? G[(long long)i * k + j] : 0.f;
+    for (int v = 0; v < LR; ++v) {
+      const int i = i0 + v * (CQ_NT / 32);
+#pragma unroll
+      for (int t = 0; t < MAX_K / 32; ++t) {
+        const int j = lane + 32 * t;
+        g[v][t] = (i < k && j <= i) ? G[(long long)i * k + j] : 0.f;
+      }
     }
 #pragma unroll
-    for (int t = 0; t < MAX_K / 32; ++t) {
-      const int j = lane + 32 * t;
-      if (j <= i) {
-        const float v = g[t] * di * d[j];
-        A[pk(i, j)] = (v == v) ? v : 0.f;
-        if (v != v) bad = 1;
+    for (int v = 0; v < LR; ++v) {
+      const int i = i0 + v * (CQ_NT / 32);
+      const float di = i < k ? d[i] : 0.f;
+#pragma unroll
+      for (int t = 0; t < MAX_K / 32; ++t) {
+        const int j = lane + 32 * t;
+        if (i < k && j <= i) {
+          const float x = g[v][t] * di * d[j];
+          A[pk(i, j)] = (x == x) ? x : 0.f;
+          if (x != x) bad = 1;
+        }
       }
     }
   }
@@ -305,36 +315,58 @@ __global__ void __launch_bounds__(CQ_NT, 1)
       const unsigned deadm = __ballot_sync(0xffffffffu, lane < pw && d[p0 + lane] == 0.f);
       unsigned brokem = 0;
       float myinv = 0.f;
-      // Per step, the pivot comes by one shuffle; the new column L_.,j goes
-      // through shared memory and is read back as float4 broadcasts (a
-      // shuffle per trailing column made each step several hundred cycles).
+      // Four columns at a time: their 4 x 4 diagonal block comes to every lane
+      // by ten shuffles and is factored by all of them alike, each lane solves
+      // its row's four entries against it, and these go through shared memory
+      // once, read back as float4 broadcasts by the trailing update.  (A column
+      // at a time the chain pivot - scaling - store - read ran 32 times, 400
+      // clocks each.)  Entries above the diagonal hold values nobody reads.
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        if (j < pw) {
-          const float piv = __shfl_sync(0xffffffffu, r[j], j);
-          const bool dead = (deadm >> j) & 1u;
-          const bool broke = !dead && !(piv > tau);
-          const float rs = rsqrtf(piv);
-          const bool good = !(dead || broke);
-          const float ljj = good ? piv * rs : 1.f;
-          const float inv = good ? rs : 0.f;
-          if (broke) brokem |= 1u << j;
-          if (lane == j) myinv = inv;
-          const float lj = r[j] * inv;   // L_lane,j (lane > j)
-          r[j] = lane == j ? ljj : (lane > j ? lj : r[j]);
-          if (j < 31) {
-            colb[lane] = lj;
+      for (int jb = 0; jb < 8; ++jb) {
+        const int j0 = 4 * jb;
+        if (j0 < pw) {
+          float l[4][4], iv[4], x[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c <= i; ++c) l[i][c] = __shfl_sync(0xffffffffu, r[j0 + c], j0 + i);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float piv = l[c][c];
+            const bool dead = ((deadm >> (j0 + c)) & 1u) || j0 + c >= pw;
+            const bool broke = !dead && !(piv > tau);
+            const float rs = rsqrtf(piv);
+            const bool good = !(dead || broke);
+            l[c][c] = good ? piv * rs : 1.f;
+            iv[c] = good ? rs : 0.f;
+            if (broke) brokem |= 1u << (j0 + c);
+#pragma unroll
+            for (int i = c + 1; i < 4; ++i) l[i][c] *= iv[c];
+#pragma unroll
+            for (int i = c + 1; i < 4; ++i)
+#pragma unroll
+              for (int k = c + 1; k <= i; ++k) l[i][k] = fmaf(-l[i][c], l[k][c], l[i][k]);
+            if (lane == j0 + c) myinv = iv[c];
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float v = r[j0 + c];
+#pragma unroll
+            for (int k = 0; k < c; ++k) v = fmaf(-x[k], l[c][k], v);
+            x[c] = v * iv[c];
+            r[j0 + c] = lane == j0 + c ? l[c][c] : (lane > j0 + c ? x[c] : r[j0 + c]);
+          }
+          if (j0 < 28) {
+            colb[lane] = make_float4(x[0], x[1], x[2], x[3]);
             __syncwarp();
-            // trailing part of the block: r[c] -= L_lane,j L_c,j for j < c <= lane
+            // trailing part of the block: r[c] -= sum of L_lane,. L_c,.
 #pragma unroll
-            for (int c4 = (j + 1) / 4; c4 < 8; ++c4) {
-              const float4 x4 = *reinterpret_cast<const float4*>(colb + 4 * c4);
-              const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int c = 4 * c4 + u;
-                if (c > j) r[c] = lane >= c ? fmaf(-lj, xs[u], r[c]) : r[c];
-              }
+            for (int c = j0 + 4; c < 32; ++c) {
+              const float4 y = colb[c];
+              r[c] = fmaf(-x[0], y.x, r[c]);
+              r[c] = fmaf(-x[1], y.y, r[c]);
+              r[c] = fmaf(-x[2], y.z, r[c]);
+              r[c] = fmaf(-x[3], y.w, r[c]);
             }
             __syncwarp();
           }
@@ -610,23 +642,26 @@ __global__ void __launch_bounds__(256)
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const int n0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const long long kk = (long long)k * k;
-  auto sum = [&](long long e) {
-    float v = 0.f;
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) v += part[s * kk + e];
-    return v;
-  };
-  // the diagonal entries of the tile's rows and columns
-  if (ty < 2) {
-    const int i = (ty ? c0 : n0) + tx;
-    (ty ? dc : dn)[tx] = i < k ? sum((long long)i * k + i) : 0.f;
-  }
-  float g[4];
+  // the thread's four entries and, in two warps, a diagonal entry of the
+  // tile's rows or columns, summed side by side
+  long long at[5];
+  bool in[5];
+  const int di = (ty ? c0 : n0) + tx;
+  at[4] = (long long)di * k + di;
+  in[4] = ty < 2 && di < k;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int n = n0 + ty + 8 * u, c = c0 + tx;
-    g[u] = (n < k && c < k) ? sum((long long)n * k + c) : 0.f;
+    at[u] = (long long)n * k + c;
+    in[u] = n < k && c < k;
   }
+  float g[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int s = 0; s < splits; ++s)
+#pragma unroll
+    for (int u = 0; u < 5; ++u)
+      if (in[u]) g[u] += part[s * kk + at[u]];
+  if (ty < 2) (ty ? dc : dn)[tx] = g[4];
   __syncthreads();
   bool big = false;
 #pragma unroll
@@ -858,34 +893,33 @@ __global__ void __launch_bounds__(256)
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const long long n = (long long)R * Cc;
-  auto sum = [&](long long e) {
-    float v = 0.f;
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) v += part[s * n + e];
-    return v;
-  };
   const bool grams = r0 + 31 >= o.r_gram || c0 + 31 >= o.c_gram;   // some Gram entry in this tile
-  if (grams && ty < 2) {
-    // Gram index of the tile's rows (ty = 0) and columns (ty = 1), and the
-    // diagonal entry there
-    const int i = ty == 0 ? r0 + tx - (o.r_gram < R ? o.r_gram : 0)
-                          : c0 + tx - (o.c_gram < Cc ? o.c_gram : 0);
-    float d = 0.f;
-    if (i >= 0 && i < o.k)
-      d = sum((long long)(i + (o.r_gram < R ? o.r_gram : 0)) * Cc + i +
-              (o.c_gram < Cc ? o.c_gram : 0));
-    (ty ? dc : dr)[tx] = d;
+  const int ro = o.r_gram < R ? o.r_gram : 0, co = o.c_gram < Cc ? o.c_gram : 0;
+  // the thread's four entries and, in two warps of a tile with Gram entries,
+  // the diagonal entry of the Gram index of the tile's rows (ty = 0) or columns
+  // (ty = 1), summed side by side
+  long long at[5];
+  bool in[5];
+  const int di = ty == 0 ? r0 + tx - ro : c0 + tx - co;
+  at[4] = (long long)(di + ro) * Cc + di + co;
+  in[4] = grams && ty < 2 && di >= 0 && di < o.k;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = r0 + ty + 8 * u, c = c0 + tx;
+    at[u] = (long long)r * Cc + c;
+    in[u] = r < R && c < Cc;
   }
+  float v4[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int s = 0; s < splits; ++s)
+#pragma unroll
+    for (int u = 0; u < 5; ++u)
+      if (in[u]) v4[u] += part[s * n + at[u]];
+  if (grams && ty < 2) (ty ? dc : dr)[tx] = v4[4];
   if (grams) __syncthreads();
   double acc = 0.0;
   float mx = 0.f;
   int live = 0;
-  float v4[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = r0 + ty + 8 * u, c = c0 + tx;
-    v4[u] = (r < R && c < Cc) ? sum((long long)r * Cc + c) : 0.f;
-  }
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int r = r0 + ty + 8 * u, c = c0 + tx;
@@ -896,7 +930,7 @@ __global__ void __launch_bounds__(256)
       o.out[(long long)r * o.ldo + c] = d;
       acc = fma(d, d, acc);
     } else {
-      const int i = r - (o.r_gram < R ? o.r_gram : 0), j = c - (o.c_gram < Cc ? o.c_gram : 0);
+      const int i = r - ro, j = c - co;
       const float gi = dr[ty + 8 * u], gj = dc[tx];
       if (i == j && gi >= 0.5f) live = 1;
       if (!(gi < 0.5f || gj < 0.5f)) {
