@@ -71,6 +71,7 @@ struct GemmF64 {
   const double* B; Idx3 bk, bn; long long sbb;
   double* C; Idx3 cm, cn; long long scb;
   double alpha, beta;
+  int sym = 0;   // C is symmetric (M = N): the upper half is mirrored from the lower
 };
 
 cudaError_t gemm_f64(const GemmF64& g, cudaStream_t st);

@@ -18,9 +18,11 @@
 //  - a warp owns 4 rows x 32 columns: rows past M cost nothing in steps of 4
 //    (the transfers have 1, 5 or 25 of them), and the two operands are
 //    exchanged when that wastes fewer lanes.
+//  - the next K-block is loaded into registers before the tile's FMAs, and a
+//    symmetric result computes only one triangle of its tiles.
 // Measured: all transfers of one observables row at L = 64, D* = 256 (31
 // GFLOP, 25 ms at the pipe's rate): 245 ms with 64 x 64 tiles and no split,
-// 38 ms with these.
+// 38.5 ms with small split tiles, 35.8 ms with the last item.
 #include "common.cuh"
 
 #include <cooperative_groups.h>
@@ -47,8 +49,12 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmF64 g, int a_kfast, int b_
                                                   int k_per) {
   __shared__ __align__(16) double As[BK][LDA];
   __shared__ __align__(16) double Bs[BK][LDB];
-  __shared__ long long offAm[BM], offBn[BN], offAk[BK], offBk[BK];
+  __shared__ long long offAm[BM], offBn[BN];
 
+  // a symmetric result: the tiles above the diagonal are mirrored (every rank of
+  // a cluster has the same tile)
+  if (g.sym && blockIdx.x > blockIdx.y) return;
+  const bool mirror = g.sym && blockIdx.x < blockIdx.y;
   const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int rank = SPLIT ? (int)(blockIdx.z % splits) : 0;
@@ -69,34 +75,33 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmF64 g, int a_kfast, int b_
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   const bool live = m0 + 4 * warp < g.M;   // this warp's rows (uniform in the warp)
 
+  // this thread's two elements of each operand's K-block; a block is loaded
+  // into registers while the one before it is multiplied
+  const int ami = a_kfast ? tid / BK : tid % BM, aki = a_kfast ? tid % BK : tid / BM;
+  const int bni = b_kfast ? tid / BK : tid % BN, bki = b_kfast ? tid % BK : tid / BN;
+  const int ams = a_kfast ? NT / BK : 0, aks = a_kfast ? 0 : NT / BM;   // step to the second
+  const int bns = b_kfast ? NT / BK : 0, bks = b_kfast ? 0 : NT / BN;
+  double va[2], vb[2];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int mi = ami + q * ams, ka = k0 + aki + q * aks;
+      const int ni = bni + q * bns, kb = k0 + bki + q * bks;
+      va[q] = (m0 + mi < g.M && ka < k_end) ? A[offAm[mi] + off32(g.ak, ka)] : 0.0;
+      vb[q] = (n0 + ni < g.N && kb < k_end) ? B[offBn[ni] + off32(g.bk, kb)] : 0.0;
+    }
+  };
+  __syncthreads();
+  if (k_begin < k_end) load(k_begin);
   for (int k0 = k_begin; k0 < k_end; k0 += BK) {
     __syncthreads();
-    if (tid < BK) {
-      const int k = k0 + tid;
-      offAk[tid] = (k < k_end) ? off32(g.ak, k) : 0;
-    } else if (tid >= 32 && tid < 32 + BK) {
-      const int k = k0 + tid - 32;
-      offBk[tid - 32] = (k < k_end) ? off32(g.bk, k) : 0;
-    }
-    __syncthreads();
-    double va[2], vb[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const int e = tid + q * NT;
-      const int mi = a_kfast ? e / BK : e % BM, ka = a_kfast ? e % BK : e / BM;
-      const int ni = b_kfast ? e / BK : e % BN, kb = b_kfast ? e % BK : e / BN;
-      va[q] = (m0 + mi < g.M && k0 + ka < k_end) ? A[offAm[mi] + offAk[ka]] : 0.0;
-      vb[q] = (n0 + ni < g.N && k0 + kb < k_end) ? B[offBk[kb] + offBn[ni]] : 0.0;
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int e = tid + q * NT;
-      const int mi = a_kfast ? e / BK : e % BM, ka = a_kfast ? e % BK : e / BM;
-      const int ni = b_kfast ? e / BK : e % BN, kb = b_kfast ? e % BK : e / BN;
-      As[ka][mi] = va[q];
-      Bs[kb][ni] = vb[q];
+      As[aki + q * aks][ami + q * ams] = va[q];
+      Bs[bki + q * bks][bni + q * bns] = vb[q];
     }
     __syncthreads();
+    if (k0 + BK < k_end) load(k0 + BK);
     if (live) {
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
@@ -124,6 +129,7 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmF64 g, int a_kfast, int b_
       double v = g.alpha * acc[i];
       if (g.beta != 0.0) v += g.beta * C[o];
       C[o] = v;
+      if (mirror) C[off32(g.cm, n) + off32(g.cn, m)] = v;
     }
     return;
   }
@@ -143,6 +149,7 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmF64 g, int a_kfast, int b_
       double v = g.alpha * s;
       if (g.beta != 0.0) v += g.beta * C[o];
       C[o] = v;
+      if (mirror) C[off32(g.cm, n) + off32(g.cn, m)] = v;
     }
   }
   cluster.sync();   // peers may still be reading this CTA's tile
@@ -186,7 +193,9 @@ cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
   // Split of the contraction: the fewest K-steps on the busiest SM.  A split
   // adds its start and the exchange of its partial tile, about two K-steps
   // (16 x 32 x 32 FMAs at 2 a clock, 4 us each); a step is one K-block of 16.
-  const long long tiles = (long long)grid.x * grid.y * g.batch;
+  if (g.sym && g.M != g.N) return cudaErrorInvalidValue;
+  const long long tiles = g.sym ? (long long)grid.x * (grid.x + 1) / 2 * g.batch
+                                : (long long)grid.x * grid.y * g.batch;
   const int kb = (g.K + BK - 1) / BK;
   int splits = 1;
   long long best = 0;

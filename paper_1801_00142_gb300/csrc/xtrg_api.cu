@@ -132,7 +132,7 @@ bool plan_sizes(int L, int DH, const xtrg_config* cfg, Plan* p) {
   t += up(2 * p->n_svd_cols * 8);           // squared column norms of the split
   t += up(p->n_usbuf * 8);
   t += 3 * up(p->n_obs * 8);
-  t += 8 * up(p->n_herm * 8);              // Hermiticity transfers: 2 + 2 ping-pong, T (x4)
+  t += 4 * up(p->n_herm * 8) + up(8 * p->n_herm * 8);   // Hermiticity transfers: 2 + 2 ping-pong, 2 T
   t += up(64 * 8);                          // scalars
   t += p->mixed_bytes;
   p->total = t;
@@ -1069,16 +1069,19 @@ xtrg_status herm_transfers(xtrg_ctx* ctx, double* fro, double* trr) {
     const int l = R.dims[i], r = R.dims[i + 1];
     double* Ef = ctx->hf[i & 1];
     double* Er = ctx->hr[i & 1];
+    // both T[m][(s,t,x)] = sum_l E[l][m] rho[l][(s,t,x)] in one launch
+    const long long ts = 4 * (long long)ctx->plan.n_herm;
+    TRY(gemm64(ctx, mk(l, 4 * r, l, 2, Ef, idx_plain(1), idx_plain(l), Er - Ef, R.site[i],
+                       idx_plain(4 * r), idx_plain(1), 0, T, idx_plain(4 * r), idx_plain(1), ts)));
     for (int which = 0; which < 2; ++which) {
-      const double* E = which == 0 ? Ef : Er;
       double* En = which == 0 ? ctx->hf[(i + 1) & 1] : ctx->hr[(i + 1) & 1];
-      // T[m][(s,t,x)] = sum_l E[l][m] rho[l][(s,t,x)]
-      TRY(gemm64(ctx, mk(l, 4 * r, l, 1, E, idx_plain(1), idx_plain(l), 0, R.site[i],
-                         idx_plain(4 * r), idx_plain(1), 0, T, idx_plain(4 * r), idx_plain(1), 0)));
-      // E'[x][y] = sum_{(m,s,t)} T[(m,s,t)][x] rho[m][s or t][t or s][y]
+      // E'[x][y] = sum_{(m,s,t)} T[(m,s,t)][x] rho[m][s or t][t or s][y], symmetric
+      // in x, y as E is in l, m (the transpose exchanges the two rho)
       const Idx3 bk = which == 0 ? idx_plain(r) : idx_split3(2, 2, 4LL * r, r, 2LL * r);
-      TRY(gemm64(ctx, mk(r, r, 4 * l, 1, T, idx_plain(1), idx_plain(r), 0, R.site[i], bk,
-                         idx_plain(1), 0, En, idx_plain(r), idx_plain(1), 0)));
+      GemmF64 g = mk(r, r, 4 * l, 1, T + which * ts, idx_plain(1), idx_plain(r), 0, R.site[i], bk,
+                     idx_plain(1), 0, En, idx_plain(r), idx_plain(1), 0);
+      g.sym = 1;
+      TRY(gemm64(ctx, g));
     }
   }
   CK(cudaMemcpyAsync(fro, ctx->hf[L & 1], sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
@@ -1169,7 +1172,7 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
     ctx->hf[i] = (double*)carve(ctx, p.n_herm * 8);
     ctx->hr[i] = (double*)carve(ctx, p.n_herm * 8);
   }
-  ctx->ht = (double*)carve(ctx, 4 * p.n_herm * 8);
+  ctx->ht = (double*)carve(ctx, 8 * p.n_herm * 8);
   ctx->scal = (double*)carve(ctx, 64 * 8);
   ok = ok && envbase && ctx->pp[0] && ctx->pp[1] && ctx->T1 && ctx->Lp && ctx->Rp && ctx->CE &&
        ctx->svd.W && ctx->svd.V && ctx->svd.sig && ctx->svd.perm && ctx->svd.nrm &&
