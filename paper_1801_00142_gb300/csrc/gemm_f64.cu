@@ -22,7 +22,8 @@
 //    symmetric result computes only one triangle of its tiles.
 // Measured: all transfers of one observables row at L = 64, D* = 256 (31
 // GFLOP, 25 ms at the pipe's rate): 245 ms with 64 x 64 tiles and no split,
-// 38.5 ms with small split tiles, 35.8 ms with the last item.
+// 38.5 ms with small split tiles, 35.8 ms with the last item, 29.0 ms with one
+// CTA an SM (see the launch).
 #include "common.cuh"
 
 #include <cooperative_groups.h>
@@ -164,6 +165,8 @@ int innermost_unit(const Idx3& d) {
 
 inline long long up_to(long long x, long long q) { return (x + q - 1) / q * q; }
 
+// Dynamic shared memory that keeps an SM to one CTA (see the launch).
+constexpr int ALONE_SMEM = 120 * 1024;
 PerDevice<int> g_sms;
 
 }  // namespace
@@ -185,6 +188,9 @@ cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
   cudaError_t e = g_sms.get(
       [](int dev) {
         int n = 0;
+        if (cudaFuncSetAttribute(gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 ALONE_SMEM) != cudaSuccess)
+          cudaGetLastError();
         return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0
                    ? n : 152;
       },
@@ -226,6 +232,11 @@ cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_kernel<true>, g, a_kfast, b_kfast, splits,
-                            (kb + splits - 1) / splits * BK);
+  // When every CTA could have an SM to itself it gets one: the CTAs of a cluster
+  // are otherwise put two to an SM, which then takes twice as long (observables
+  // row: 35.8 ms, 29.0 ms with this).  Short ones are launch-bound either way
+  // and keep their small footprint for the kernels of other streams.
+  const int blocks = (kb + splits - 1) / splits;
+  if (tiles * splits <= sms && blocks >= 4) cfg.dynamicSmemBytes = ALONE_SMEM;
+  return cudaLaunchKernelEx(&cfg, gemm_kernel<true>, g, a_kfast, b_kfast, splits, blocks * BK);
 }
