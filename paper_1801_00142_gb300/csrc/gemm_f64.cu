@@ -23,7 +23,7 @@
 // Measured: all transfers of one observables row at L = 64, D* = 256 (31
 // GFLOP, 25 ms at the pipe's rate): 245 ms with 64 x 64 tiles and no split,
 // 38.5 ms with small split tiles, 35.8 ms with the last item, 29.0 ms with one
-// CTA an SM (see the launch).
+// CTA an SM (see the launch), 28.0 ms with the present rule for the split.
 #include "common.cuh"
 
 #include <cooperative_groups.h>
@@ -199,6 +199,8 @@ cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
   // Split of the contraction: the fewest K-steps on the busiest SM.  A split
   // adds its start and the exchange of its partial tile, about two K-steps
   // (16 x 32 x 32 FMAs at 2 a clock, 4 us each); a step is one K-block of 16.
+  // It adds them once: with several CTAs an SM the others compute meanwhile
+  // (counted for each of them: observables row 29.0 ms, once: 28.0 ms).
   if (g.sym && g.M != g.N) return cudaErrorInvalidValue;
   const long long tiles = g.sym ? (long long)grid.x * (grid.x + 1) / 2 * g.batch
                                 : (long long)grid.x * grid.y * g.batch;
@@ -206,8 +208,7 @@ cudaError_t gemm_f64(const GemmF64& g0, cudaStream_t st) {
   int splits = 1;
   long long best = 0;
   for (int s = 1; s <= SPLIT_MAX && (s == 1 || (s <= kb && g.batch * s <= 65535)); s *= 2) {
-    const long long per = (kb + s - 1) / s + (s > 1 ? 2 : 0);
-    const long long cost = (tiles * s + sms - 1) / sms * per;
+    const long long cost = (tiles * s + sms - 1) / sms * ((kb + s - 1) / s) + (s > 1 ? 2 : 0);
     if (s == 1 || cost < best) {
       best = cost;
       splits = s;
