@@ -3,13 +3,14 @@
 // CTA tile 128 x 128 (M x N), K-block of 64 BF16 (one 128-byte swizzle row;
 // 2 stages at 6 planes); persistent CTAs (one per SM).  Warp 0: TMA producer (one elected thread);
 // warp 1: MMA issuer (one elected thread, 4 x UMMA_K=16 per K-block and
-// product); warp 2: tensor-memory allocation; warps 4-11: epilogue
-// (tcgen05.ld 32x32b, lane quarter = warp % 4, half of the columns each).
+// product); warp 2: tensor-memory allocation; warps 4 on: epilogue
+// (tcgen05.ld 32x32b, lane quarter = warp % 4, a part of the columns each).
 // With four epilogue warps, each storing its own rows, the epilogue bound every
 // site of short contraction: at L = 64, D* = 256 the first substep ran at 116
 // TFLOP/s algorithmic and the second at 192, with eight and the store forms of
 // store_chunk at 161 and 222 (C_E, whose K hides it: 257); an odd bond of 173 in
-// two planes 25 -> 52 and 104 -> 137, its environment update 35 -> 91.
+// two planes 25 -> 52 and 104 -> 137, its environment update 35 -> 91 (16 warps
+// took that doubling a further 13 % down: see Epi).
 //
 // Accumulation.  The tensor core rounds its FP32 accumulator toward zero, so
 // long accumulation chains in tensor memory shrink every output by a
@@ -37,9 +38,19 @@
 namespace {
 
 constexpr int BM = 128, BN = 128;
-constexpr int EPI_WARPS = 8;                 // warps 4..11
-constexpr int EPI_COLS = BN * 4 / EPI_WARPS;   // output columns of each
-constexpr int NTHREADS = 128 + 32 * EPI_WARPS;
+// Epilogue warps (from warp 4 on) by number of plane products: a K-block of
+// three takes the tensor cores half the time of one of six, so its tiles need
+// the faster epilogue.  A doubling at L = 20, D* = 173 in three products: 47.8
+// ms with 8 warps, 41.6 with 16; one at L = 64, D* = 256 in six: 715 ms with 8,
+// 733 with 16.
+template <int NPROD>
+struct Epi {
+  static constexpr int WARPS = NPROD > 3 ? 8 : 16;
+  static constexpr int COLS = BN * 4 / WARPS;      // output columns of each
+  static constexpr int THREADS = 128 + 32 * WARPS;
+  static constexpr int STAGED = COLS / 2;          // columns staged at a time (see store_chunk)
+  static constexpr int STG = STAGED * 2 + 16;      // bytes of a staged row: padded, 16-byte aligned
+};
 
 // Shared-memory geometry for a K-block of BK BF16 (64: 128-byte swizzle,
 // 32: 64-byte swizzle).  K-major tiles are BM rows of SW bytes in 8-row
@@ -193,15 +204,16 @@ __device__ __forceinline__ void tmem_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// acc[0..EPI_COLS) += the accumulator columns at taddr, round-to-nearest; all
+// acc[0..COLS) += the accumulator columns at taddr, round-to-nearest; all
 // loads in flight before the one wait
+template <int COLS>
 __device__ __forceinline__ void tmem_add(uint32_t taddr, float* acc) {
-  uint32_t r[EPI_COLS];
+  uint32_t r[COLS];
 #pragma unroll
-  for (int c = 0; c < EPI_COLS; c += 32) tmem_ld32(taddr + (uint32_t)c, r + c);
+  for (int c = 0; c < COLS; c += 32) tmem_ld32(taddr + (uint32_t)c, r + c);
   tmem_wait();
 #pragma unroll
-  for (int c = 0; c < EPI_COLS; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(r[c]));
+  for (int c = 0; c < COLS; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(r[c]));
 }
 
 __device__ __forceinline__ void store_out(const TcOutput& o, long long off, float v) {
@@ -252,8 +264,9 @@ struct ChunkForm {
   int layout;        // columns: 2 contiguous, 1 paired, 0 other
   bool rows_adjacent, rowpair;
 };
-constexpr int STG = 80;   // bytes of a staged row: 32 BF16, padded, 16-byte aligned
 
+// SW: columns turned at a time
+template <int SW>
 __device__ __forceinline__ void store_chunk(const TcOutput& o, long long om, bool valid,
                                             const long long* col, const ChunkForm& f, int ncols,
                                             const float* v, uint8_t* stage) {
@@ -309,41 +322,49 @@ __device__ __forceinline__ void store_chunk(const TcOutput& o, long long om, boo
   const unsigned vm = __ballot_sync(0xffffffffu, valid);
   const bool vec = f.layout == 2 && ncols == 32 && (ps & 7) == 0 &&
                    __all_sync(0xffffffffu, !valid || ((om + col[0]) & 7) == 0);
-  const long long mycol = lane < ncols ? col[lane] : 0;
+  constexpr int STG = SW * 2 + 16, C8 = SW / 8, RPI = 32 / SW;
+  long long mycol[32 / SW];
+#pragma unroll
+  for (int h = 0; h < 32; h += SW) mycol[h / SW] = h + lane % SW < ncols ? col[h + lane % SW] : 0;
   for (int q = 0; q < o.planes; ++q) {
-    // this lane's row of plane q
-#pragma unroll
-    for (int q8 = 0; q8 < 4; ++q8) {
-      uint32_t w[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t w0, w1, w2;
-        split_pack2(v[q8 * 8 + 2 * e], v[q8 * 8 + 2 * e + 1], w0, w1, w2);
-        w[e] = q == 0 ? w0 : (q == 1 ? w1 : w2);
-      }
-      *reinterpret_cast<uint4*>(stage + lane * STG + q8 * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-    __syncwarp();
     __nv_bfloat16* out = o.bf16 + q * ps;
-    if (vec) {
-      const long long c0 = col[0];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = i * 8 + lane / 4;
-        const long long omr = __shfl_sync(0xffffffffu, om, r);
-        if ((vm >> r) & 1)
-          *reinterpret_cast<uint4*>(out + omr + c0 + (lane % 4) * 8) =
-              *reinterpret_cast<const uint4*>(stage + r * STG + (lane % 4) * 16);
+    for (int h = 0; h < 32; h += SW) {
+      // this lane's row of plane q
+#pragma unroll
+      for (int q8 = 0; q8 < C8; ++q8) {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          uint32_t w0, w1, w2;
+          split_pack2(v[h + q8 * 8 + 2 * e], v[h + q8 * 8 + 2 * e + 1], w0, w1, w2);
+          w[e] = q == 0 ? w0 : (q == 1 ? w1 : w2);
+        }
+        *reinterpret_cast<uint4*>(stage + lane * STG + q8 * 16) = make_uint4(w[0], w[1], w[2], w[3]);
       }
-    } else {
+      __syncwarp();
+      if (vec) {
+        const long long c0 = col[0] + h;
+#pragma unroll
+        for (int i = 0; i < C8; ++i) {
+          const int r = i * (32 / C8) + lane / C8;
+          const long long omr = __shfl_sync(0xffffffffu, om, r);
+          if ((vm >> r) & 1)
+            *reinterpret_cast<uint4*>(out + omr + c0 + (lane % C8) * 8) =
+                *reinterpret_cast<const uint4*>(stage + r * STG + (lane % C8) * 16);
+        }
+      } else {
 #pragma unroll 4
-      for (int r = 0; r < 32; ++r) {
-        const long long omr = __shfl_sync(0xffffffffu, om, r);
-        if (((vm >> r) & 1) && lane < ncols)
-          out[omr + mycol] = *reinterpret_cast<const __nv_bfloat16*>(stage + r * STG + lane * 2);
+        for (int i = 0; i < SW; ++i) {
+          const int r = i * RPI + lane / SW;
+          const long long omr = __shfl_sync(0xffffffffu, om, r);
+          if (((vm >> r) & 1) && h + lane % SW < ncols)
+            out[omr + mycol[h / SW]] =
+                *reinterpret_cast<const __nv_bfloat16*>(stage + r * STG + (lane % SW) * 2);
+        }
       }
+      __syncwarp();
     }
-    __syncwarp();
   }
 }
 
@@ -378,10 +399,11 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 // descriptors plus compile-time offsets (measured: the runtime-selected
 // descriptors alone cost 16 % of the kernel's time).
 template <int BK, int BMN, int NPROD>
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __launch_bounds__(Epi<NPROD>::THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                    const KParams p) {
   using G = Geo<BK>;
+  using E = Epi<NPROD>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -395,7 +417,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* corr_empty = corr_full + 2; // [2]
   uint64_t* done = corr_empty + 2;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
-  long long* col_off_all = (long long*)(tmem_slot + 2);   // [EPI_WARPS][EPI_COLS] column offsets
+  long long* col_off_all = (long long*)(tmem_slot + 2);   // [warps][columns of each] offsets
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int tiles_n = (p.N + BN - 1) / BN, tiles_m = (p.M + BM - 1) / BM;
@@ -410,9 +432,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&main_full[b], 1);
-      mbar_init(&main_empty[b], EPI_WARPS);
+      mbar_init(&main_empty[b], E::WARPS);
       mbar_init(&corr_full[b], 1);
-      mbar_init(&corr_empty[b], EPI_WARPS);
+      mbar_init(&corr_empty[b], E::WARPS);
     }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -534,13 +556,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     mma_commit(done);
   } else if (warp >= 4) {
     // ---------------- epilogue (warp % 4 selects the TMEM lane quarter, two
-    // warps share it, each with half of the columns: one warp per scheduler
+    // or four warps share it, each with its columns: one warp per scheduler
     // could not hide its own latencies, and short-K tiles waited for it)
+    constexpr int EPI_COLS = E::COLS;
     const int q = warp % 4, ec0 = (warp - 4) / 4 * EPI_COLS;
     const TcOutput& o = p.out;
     long long* col_off = col_off_all + (warp - 4) * EPI_COLS;
     uint8_t* stage = (uint8_t*)(((uintptr_t)(col_off_all + 4 * BN) + 15) & ~(uintptr_t)15) +
-                     (warp - 4) * 32 * STG;
+                     (warp - 4) * 32 * E::STG;
     const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ec0;
     long long h = 0;   // main chunks drained
     int j = 0;
@@ -588,7 +611,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         ok = mbar_wait(&main_full[mb], (uint32_t)((h >> 1) & 1), p.err);
         if (!ok) break;
         fence_after();
-        tmem_add(lane_base + (uint32_t)(mb * BN), acc);
+        tmem_add<EPI_COLS>(lane_base + (uint32_t)(mb * BN), acc);
         fence_before();
         __syncwarp();
         if (lane == 0)
@@ -600,7 +623,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         ok = mbar_wait(&corr_full[cb], (uint32_t)((j >> 1) & 1), p.err);
         if (!ok) break;
         fence_after();
-        if (kb_end > kb_begin) tmem_add(lane_base + (uint32_t)(CORR_COL + cb * BN), acc);
+        if (kb_end > kb_begin) tmem_add<EPI_COLS>(lane_base + (uint32_t)(CORR_COL + cb * BN), acc);
         fence_before();
         __syncwarp();
         if (lane == 0)
@@ -629,7 +652,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // whole where its lanes trade values)
       if (!__any_sync(0xffffffffu, valid) || (o.mode >= TC_OUT_PARTIAL && !valid)) continue;
       const float alpha = (float)o.alpha;
-      // the two chunks in a loop that is not unrolled: the store forms are long,
+      // the chunks in a loop that is not unrolled: the store forms are long,
       // and a tile's time is what a few warps need to fetch and run them
 #pragma unroll 1
       for (int ch = 0; ch < EPI_COLS / 32; ++ch) {
@@ -672,7 +695,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
           for (int jj = 0; jj < 32; ++jj) v[jj] *= alpha;
           form.layout = (layouts >> (2 * ch)) & 3;
-          store_chunk(o, om, valid, col_off + c, form, ncols, v, stage);
+          store_chunk<E::STAGED>(o, om, valid, col_off + c, form, ncols, v, stage);
         }
       }
     }
@@ -785,6 +808,15 @@ cudaError_t make_map(CUtensorMap* map, const TcOperand& op, int BK) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+template <int BMN, int NPROD>
+void launch(dim3 grid, cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
+            const KParams& p, int stage_bytes) {
+  using E = Epi<NPROD>;
+  const int smem = p.stages * stage_bytes + 1024 + (2 * p.stages + 9) * 8 + 8 + 4 * BN * 8 + 64 +
+                   E::WARPS * 32 * E::STG;
+  tc_gemm_kernel<K_BLOCK, BMN, NPROD><<<grid, E::THREADS, smem, st>>>(ma, mb, p);
+}
+
 }  // namespace
 
 cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K, int batch,
@@ -830,7 +862,6 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K,
   cudaError_t e;
   if ((e = make_map(&ma, A, BK)) != cudaSuccess) return e;
   if ((e = make_map(&mb, B, BK)) != cudaSuccess) return e;
-  const int smem = S * stage_bytes + 1024 + (2 * S + 9) * 8 + 8 + 4 * BN * 8 + 64 + EPI_WARPS * 32 * STG;
   int sms = 0;
   if ((e = launch_setup(&sms)) != cudaSuccess) return e;
   const long long tiles =
@@ -840,12 +871,12 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K,
   note_launch();
   const int sel = (B.mn_major ? 3 : 0) + (nprod == 1 ? 0 : nprod == 3 ? 1 : 2);
   switch (sel) {
-    case 0: tc_gemm_kernel<K_BLOCK, 0, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 1: tc_gemm_kernel<K_BLOCK, 0, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 2: tc_gemm_kernel<K_BLOCK, 0, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 3: tc_gemm_kernel<K_BLOCK, 1, 1><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    case 4: tc_gemm_kernel<K_BLOCK, 1, 3><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
-    default: tc_gemm_kernel<K_BLOCK, 1, 6><<<grid, NTHREADS, smem, st>>>(ma, mb, p); break;
+    case 0: launch<0, 1>(grid, st, ma, mb, p, stage_bytes); break;
+    case 1: launch<0, 3>(grid, st, ma, mb, p, stage_bytes); break;
+    case 2: launch<0, 6>(grid, st, ma, mb, p, stage_bytes); break;
+    case 3: launch<1, 1>(grid, st, ma, mb, p, stage_bytes); break;
+    case 4: launch<1, 3>(grid, st, ma, mb, p, stage_bytes); break;
+    default: launch<1, 6>(grid, st, ma, mb, p, stage_bytes); break;
   }
   return cudaGetLastError();
 }
