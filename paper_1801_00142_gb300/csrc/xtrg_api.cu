@@ -90,7 +90,7 @@ bool plan_sizes(int L, int DH, const xtrg_config* cfg, Plan* p) {
   p->n_svd_cols = 4 * capc;
   p->n_usbuf = capc * capc;
   p->n_obs = (size_t)DH * DH * 4 * cap * 2;
-  p->n_herm = cap * cap;   // one transfer matrix of the Hermiticity check (T: 4 of these)
+  p->n_herm = cap * cap;   // one transfer matrix of the Hermiticity check
   p->planes = cfg->prec == XTRG_BF16X6 ? 3 : 2;
   {
     const size_t c = cap, l1 = tc_ld(c), l2 = tc_ld(2 * c), lsq = tc_ld(c * c), l4 = tc_ld(4 * c);
@@ -129,10 +129,9 @@ bool plan_sizes(int L, int DH, const xtrg_config* cfg, Plan* p) {
   t += 3 * up(p->n_part * 8);               // T1, Lpart, Rpart
   t += up(p->n_ce * 8);                     // C_E
   t += 2 * up(p->n_svd * 8) + up(p->n_svd_cols * 8) + up(p->n_svd_cols * 4) + 3 * ALIGN;
-  t += up(2 * p->n_svd_cols * 8);           // squared column norms of the split
   t += up(p->n_usbuf * 8);
   t += 3 * up(p->n_obs * 8);
-  t += 4 * up(p->n_herm * 8) + up(8 * p->n_herm * 8);   // Hermiticity transfers: 2 + 2 ping-pong, 2 T
+  t += 4 * up(p->n_herm * 8);               // Hermiticity transfers: 2 + 2 ping-pong
   t += up(64 * 8);                          // scalars
   t += p->mixed_bytes;
   p->total = t;
@@ -1160,7 +1159,6 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
   ctx->svd.V = (double*)carve(ctx, p.n_svd * 8);
   ctx->svd.sig = (double*)carve(ctx, p.n_svd_cols * 8);
   ctx->svd.perm = (int*)carve(ctx, p.n_svd_cols * 4);
-  ctx->svd.nrm = (double*)carve(ctx, 2 * p.n_svd_cols * 8);
   ctx->svd.counter = (int*)carve(ctx, 32);
   ctx->svd.kept = (int*)carve(ctx, 16);
   ctx->svd.stats = (double*)carve(ctx, 64);
@@ -1172,7 +1170,11 @@ extern "C" xtrg_status xtrg_create(xtrg_ctx** out, const xtrg_mpo* Hm, const xtr
     ctx->hf[i] = (double*)carve(ctx, p.n_herm * 8);
     ctx->hr[i] = (double*)carve(ctx, p.n_herm * 8);
   }
-  ctx->ht = (double*)carve(ctx, 8 * p.n_herm * 8);
+  // two uses of a buffer that never meet: the squared column norms of a split (2
+  // n_svd_cols <= n_obs) and the transfers of the traces; the transfers' T (two of
+  // 4 n_herm <= n_ce) and C_E
+  ctx->svd.nrm = ctx->ob[2];
+  ctx->ht = ctx->CE;
   ctx->scal = (double*)carve(ctx, 64 * 8);
   ok = ok && envbase && ctx->pp[0] && ctx->pp[1] && ctx->T1 && ctx->Lp && ctx->Rp && ctx->CE &&
        ctx->svd.W && ctx->svd.V && ctx->svd.sig && ctx->svd.perm && ctx->svd.nrm &&
