@@ -37,8 +37,8 @@
 // of FP64 (two FMAs a clock each), run as a cooperative grid with a bounded
 // barrier (on expiry the kernel records a timeout and every CTA leaves).
 // Measured, one FP64 doubling at L = 32, D* = 40, one sweep (62 splits of up
-// to 160 x 160): 988 ms with Jacobi on C_E, 114 ms with this split (an average
-// split of its bulk takes 0.7 ms: 90 QR steps and some 400 rounds).
+// to 160 x 160): 965 ms with Jacobi on C_E, 108 ms with this split (an average
+// split of its bulk takes 0.66 ms: 90 QR steps and some 400 rounds).
 #include <math.h>
 
 #include "common.cuh"
