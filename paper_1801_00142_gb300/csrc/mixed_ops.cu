@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 
 #include "mixed_ops.cuh"
+#include "plane_layout.h"
 #include "planes.cuh"
 
 namespace {
@@ -269,12 +270,12 @@ cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int ro
 cudaError_t to_planes_pair(const double* a, int rows_a, int Ka, __nv_bfloat16* out_a, const double* b,
                            int rows_b, int Kb, __nv_bfloat16* out_b, int batch, int planes,
                            int* clear, cudaStream_t st) {
-  const long long lda = (Ka + 7) / 8 * 8, ldb = (Kb + 7) / 8 * 8;
+  const PlaneLayout la = plane_layout(rows_a, Ka, batch), lb = plane_layout(rows_b, Kb, batch);
   return launch_to_planes(
-      plane_job(a, idx_plain(Ka), idx_plain(1), (long long)rows_a * Ka, rows_a, Ka, batch, out_a, lda,
-                rows_a * lda, batch * rows_a * lda),
-      plane_job(b, idx_plain(Kb), idx_plain(1), (long long)rows_b * Kb, rows_b, Kb, batch, out_b, ldb,
-                rows_b * ldb, batch * rows_b * ldb),
+      plane_job(a, idx_plain(Ka), idx_plain(1), (long long)rows_a * Ka, rows_a, Ka, batch, out_a,
+                la.ld, la.batch_stride, la.plane_stride),
+      plane_job(b, idx_plain(Kb), idx_plain(1), (long long)rows_b * Kb, rows_b, Kb, batch, out_b,
+                lb.ld, lb.batch_stride, lb.plane_stride),
       planes, clear, st);
 }
 

@@ -9,8 +9,8 @@
 cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                       int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                       long long ops, cudaStream_t st);
-// to_planes of two batches of row-major matrices (rows x K, rows padded to a
-// multiple of 8) in one launch; *clear (may be null) is set to zero.
+// to_planes of two batches of row-major matrices (rows x K) into the layout of
+// plane_layout.h in one launch; *clear (may be null) is set to zero.
 cudaError_t to_planes_pair(const double* a, int rows_a, int Ka, __nv_bfloat16* out_a, const double* b,
                            int rows_b, int Kb, __nv_bfloat16* out_b, int batch, int planes,
                            int* clear, cudaStream_t st);

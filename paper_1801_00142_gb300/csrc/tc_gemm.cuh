@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "plane_layout.h"
 
 enum TcOutMode {
   TC_OUT_F32 = 0,      // FP32 values scattered through (cm, cn, scb)
@@ -49,6 +50,3 @@ struct TcOutput {
 // nprod in {1, 3, 6}; splitk >= 1 (only with TC_OUT_PARTIAL).
 cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K, int batch,
                     int nprod, int splitk, const TcOutput& out, int* dev_err, cudaStream_t st);
-
-// Rows needed in the padded row stride of an operand buffer with k columns.
-static inline long long tc_ld(long long k) { return (k + 7) / 8 * 8; }

@@ -1925,10 +1925,10 @@ extern "C" xtrg_status xtrg_set_graphs(xtrg_ctx* ctx, int on) {
 // partials, error flag.
 TcGemmScratch tc_gemm_scratch(int M, int N, int K, int batch, int planes, int splitk, bool b_kn) {
   TcGemmScratch w;
-  const size_t ld = (size_t)tc_ld(K);
-  w.a = up((size_t)planes * batch * M * ld * 2);
-  w.b = b_kn ? up((size_t)planes * batch * K * tc_ld(N) * 2)
-             : up((size_t)planes * batch * N * ld * 2);
+  const PlaneLayout a = plane_layout(M, K, batch);
+  const PlaneLayout b = b_kn ? plane_layout(K, N, batch) : plane_layout(N, K, batch);
+  w.a = up((size_t)planes * a.plane_stride * 2);
+  w.b = up((size_t)planes * b.plane_stride * 2);
   w.part = up((size_t)splitk * batch * M * N * 4);
   w.total = w.a + w.b + w.part + ALIGN;
   return w;
@@ -1969,18 +1969,15 @@ xtrg_status tc_gemm_run(const double* A, const double* B, double* C, int M, int 
   __nv_bfloat16* pb = (__nv_bfloat16*)(base + w.a);
   float* part = (float*)(base + w.a + w.b);
   int* err = (int*)(base + w.a + w.b + w.part);
-  const long long ld = tc_ld(K);
-  const long long ldn = tc_ld(N);
-  const long long psA = (long long)batch * M * ld;
-  const long long psB = b_kn ? (long long)batch * K * ldn : (long long)batch * N * ld;
+  const PlaneLayout la = plane_layout(M, K, batch);
+  const PlaneLayout lb = b_kn ? plane_layout(K, N, batch) : plane_layout(N, K, batch);
   // both operands' planes (B: its rows of K, K-major, or its own K x N rows,
   // MN-major) and the cleared error flag in one launch
   if ((b_kn ? to_planes_pair(A, M, K, pa, B, K, N, pb, batch, planes, err, st)
             : to_planes_pair(A, M, K, pa, B, N, K, pb, batch, planes, err, st)) != cudaSuccess)
     return XTRG_ECUDA;
-  TcOperand oa{pa, planes, M, K, ld, (long long)M * ld, psA, batch};
-  TcOperand ob{pb, planes, N, K, ld, (long long)N * ld, psB, batch};
-  if (b_kn) ob = TcOperand{pb, planes, N, K, ldn, (long long)K * ldn, psB, batch, 1};
+  const TcOperand oa{pa, planes, M, K, la.ld, la.batch_stride, la.plane_stride, batch};
+  const TcOperand ob{pb, planes, N, K, lb.ld, lb.batch_stride, lb.plane_stride, batch, b_kn ? 1 : 0};
   TcOutput out;
   memset(&out, 0, sizeof out);
   out.mode = splitk == 1 ? TC_OUT_F64 : TC_OUT_PARTIAL;
