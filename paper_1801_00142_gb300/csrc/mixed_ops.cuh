@@ -5,7 +5,9 @@
 #include "common.cuh"
 
 // out[b][r][k] = split planes of src[b*sbs + off(rv, r) + off(kv, k)] for
-// k < K, zero for K <= k < ld; planes = 2 or 3, plane stride ops.
+// k < K, zero for K <= k < ld; planes = 2 or 3, plane stride ops.  Rows are
+// stored 16 bytes at a time: out 16-byte aligned and ld, obs, ops multiples of
+// 8, else cudaErrorInvalidValue (to_planes_if and to_planes_f32 alike).
 cudaError_t to_planes(const double* src, Idx3 rv, Idx3 kv, long long sbs, int rows, int K,
                       int batch, __nv_bfloat16* out, long long ld, long long obs, int planes,
                       long long ops, cudaStream_t st);

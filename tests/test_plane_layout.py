@@ -65,3 +65,41 @@ def test_scratch_holds_the_planes_of_that_layout(nn, M, N, K, batch, planes):
     n = size(M, N, K, batch, planes, 1)
     need = a + b + batch * M * N * 4 + 4
     assert need <= n < need + 4 * 256
+
+
+REFUSE = r"""
+#include <stdio.h>
+#include "mixed_ops.cu"
+unsigned long long g_xtrg_launches;
+thread_local unsigned long long t_xtrg_launches;
+int main() {
+  struct { size_t out; long long ld, obs, ops; } c[] = {
+      {256, 9, 0, 96}, {256, 16, 56, 196}, {256, 16, 60, 192}, {264, 16, 64, 192}};
+  const Idx3 u = idx_plain(1), w = idx_plain(9);
+  for (auto& x : c) {
+    __nv_bfloat16* out = (__nv_bfloat16*)x.out;
+    printf("%d %d %d\n",
+           (int)to_planes((const double*)256, w, u, 36, 4, 9, 3, out, x.ld, x.obs, 2, x.ops, 0),
+           (int)to_planes_f32((const float*)256, w, u, 36, 4, 9, 3, out, x.ld, x.obs, 2, x.ops, 0),
+           x.obs ? 1 : (int)to_planes_if((const double*)256, w, u, 4, 9, out, x.ld, 2, x.ops,
+                                         (const double*)256, 0.0, 0));
+  }
+}
+"""
+
+
+def test_unaligned_plane_layouts_are_refused(tmp_path):
+    """A thread stores eight columns at a time, so a row stride, batch stride,
+    plane stride or start that is no multiple of 16 bytes would write past the
+    rows: the host refuses it (cudaErrorInvalidValue = 1), nothing is launched."""
+    from paper_1801_00142_gb300.build import ARCH, nvcc
+    try:
+        cc = nvcc()
+    except RuntimeError:
+        pytest.skip("no nvcc")
+    src, exe = tmp_path / "refuse.cu", tmp_path / "refuse"
+    src.write_text(REFUSE)
+    subprocess.run([cc, *ARCH, "-std=c++17", "-cudart", "shared", f"-I{CSRC}", str(src), "-o", str(exe),
+                    "-Xlinker", "-rpath,/usr/local/cuda/lib64"], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, check=True)
+    assert r.stdout.split() == ["1"] * 12
