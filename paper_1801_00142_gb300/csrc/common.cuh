@@ -82,8 +82,10 @@ cudaError_t gemm_f64(const GemmF64& g, cudaStream_t st);
 // on its triangular factor), with selection of the largest singular values.
 // See svd_jacobi.cu.
 struct SvdBuffers {
-  double* W;       // R^T of the pivoted QR, rotated: min(m, n) columns, contiguous
-  double* V;       // the columns of the split matrix, contiguous
+  double* W;       // R^T of the pivoted QR, rotated: min(m, n) columns, contiguous;
+                   // then the projection
+  double* V;       // the columns of the split matrix, contiguous; then the Gram of
+                   // the isometry
   double* nrm;     // 2 x max_cols squared column norms
   double* sig;     // ncols
   int* perm;       // ncols: perm[r] = column with the r-th largest sigma
