@@ -14,9 +14,15 @@
 //     only R^T (p x r) is formed, Q is never needed.  It ends early at rank r
 //     when what is left has a Frobenius norm below a tenth of rel_tol *
 //     sigma_max (those singular values are numerically zero), or, when kcap
-//     cuts the spectrum, below 1e-6 of what was left after kcap columns: the
-//     remainder E is orthogonal to Q, so A^T A = R^T R + E^T E and the kept
-//     subspace changes by the square of that ratio.
+//     cuts the spectrum, as soon as what is left, E, no longer counts.  E is
+//     orthogonal to Q, so A^T A = R^T R + E^T E: leaving it out loses at most
+//     |E|^2 of captured weight, and turns the kept subspace by |E|^2 over the
+//     gap of the squares at the cut, where rounding turns it by eps sigma_max
+//     over the gap.  Hence |E|^2 <= 1e-12 of the weight left after kcap columns
+//     and <= eps sigma_max sigma_k (the latter is the tighter one on flat
+//     spectra: with the first alone, values 1e-5 apart at the cut and one of
+//     9e-7 behind it gave factors off by 4e-9, now 3e-11; thermal states meet
+//     both a column or two apart).
 //  2. One-sided Jacobi orthogonalises the r columns of R^T: R^T J = X Sigma
 //     with X the wanted singular vectors.  The triangular factor of a pivoted
 //     QR is close to having orthogonal rows, and the rotations resolve small
@@ -355,7 +361,7 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
   // clocks and a warp in 64, so the sums over lanes and the scalars count
   int r = 0;
   double scale = 1.0, rem = 0.0;
-  float mx0 = 0.f, rho_k = -1.f, remf = 0.f;   // weights relative to 2^(e0 - 1023) in FP32
+  float mx0 = 0.f, remcut = -1.f, remf = 0.f;   // weights relative to 2^(e0 - 1023) in FP32
   const int e0 = biased_exp(fro);
   const float nstop = (float)(0.01 * a.rel_tol * a.rel_tol);
   const int grp = lane / LGQ, gl = lane % LGQ;
@@ -395,8 +401,9 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
       scale = ldexp(1.0, -(ilogb(bn) / 2));
     }
     if (best <= 0 || remf <= nstop * mx0) break;
-    if (j == a.kcap) rho_k = remf;
-    if (rho_k >= 0.f && j > a.kcap && remf <= 1e-12f * rho_k) break;
+    // sigma_max and sigma_k as the first pivot and the one after kcap columns show them
+    if (j == a.kcap) remcut = fminf(1e-12f * remf, 2.2e-16f * sqrtf(mx0 * scaled_float(bn, e0)));
+    if (j > a.kcap && remf <= remcut) break;
     // 1 / |pivot|: FP32 for the mantissa (in [1, 4), even exponent), then one
     // third-order step
     const int eb = biased_exp(bn), h = (eb - 1023) >> 1;   // bn = m 4^h
