@@ -90,8 +90,9 @@ struct SvdBuffers {
   double* sig;     // ncols
   int* perm;       // ncols: perm[r] = column with the r-th largest sigma
   int* counter;    // 8 words: grid barrier, rotations and unconverged pairs per sweep
-  double* stats;   // [0] = total weight, [1] = discarded fraction, [2] = sigma_max, [3] = rank
-  int* kept;       // number kept
+  double* stats;   // 8: [0] total weight, [1] discarded fraction, [2] sigma_max,
+                   // [3] ||M||_F^2, [4] columns of the QR
+  int* kept;       // 4 words: number kept, rank, sweeps, status
   size_t max_elems;   // capacity of W and of V in doubles
   int max_cols;
 };
@@ -104,6 +105,7 @@ enum SplitMode { SPLIT_RIGHT = 0, SPLIT_LEFT = 1 };
 struct SvdResult {
   int k;              // kept singular values
   int rank;           // singular values above rel_tol * sigma_max (before the cap)
+  int columns;        // columns of the pivoted QR, which the sweeps run over
   int sweeps;         // Jacobi sweeps used
   double discarded;   // discarded weight / total weight
   double sigma_max;

@@ -80,7 +80,7 @@ struct SvdArgs {
   int* cnt;           // [0..2] rotations per sweep (ring), [3..5] unconverged pairs per check (ring)
   int* out;           // [0] k, [1] rank, [2] sweeps, [3] status (0 ok, 1 timeout, 2 not converged)
   double* stats;      // [0] total weight, [1] discarded fraction, [2] sigma_max,
-                      // [3] ||M||_F^2 (accumulated while loading)
+                      // [3] ||M||_F^2 (accumulated while loading), [4] columns of the QR
   // device-decided mode (all null otherwise): run only if *run_if > thresh
   // or is not finite; keep exactly min(kcap, p, q); report into acc
   const double* run_if;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
       a.out[1] = 0;
       a.out[2] = 0;
       a.stats[0] = a.stats[2] = fro;
-      a.stats[1] = 0.0;
+      a.stats[1] = a.stats[4] = 0.0;
       if (a.run_if && a.acc.runs) atomicAdd(a.acc.runs, 1ull);
       if (a.run_if && a.acc.status) atomicMax(a.acc.status, 3);
     }
@@ -595,6 +595,7 @@ __global__ void __launch_bounds__(NT) svd_split_kernel(SvdArgs a) {
       a.stats[0] = (keptw + dropw) / scale / scale;
       a.stats[1] = keptw + dropw > 0.0 ? dropw / (keptw + dropw) : 0.0;
       a.stats[2] = smx / scale;
+      a.stats[4] = r;
       if (a.run_if) {
         if (a.acc.disc_max)
           atomicMax(reinterpret_cast<unsigned long long*>(a.acc.disc_max),
@@ -758,7 +759,7 @@ cudaError_t svd_split_f64(const double* M, int m, int n, int kcap, double rel_to
                              SvdDeviceAcc{nullptr, nullptr, nullptr});
   if (e != cudaSuccess) return e;
   int out[4];
-  double stats[3];
+  double stats[5];
   if ((e = cudaMemcpyAsync(out, buf.kept, sizeof out, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
     return e;
   if ((e = cudaMemcpyAsync(stats, buf.stats, sizeof stats, cudaMemcpyDeviceToHost, st)) !=
@@ -772,5 +773,6 @@ cudaError_t svd_split_f64(const double* M, int m, int n, int kcap, double rel_to
   res->sweeps = out[2];
   res->discarded = stats[1];
   res->sigma_max = stats[2];
+  res->columns = (int)stats[4];
   return cudaSuccess;
 }

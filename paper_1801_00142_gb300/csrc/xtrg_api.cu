@@ -298,8 +298,14 @@ xtrg_status split(xtrg_ctx* ctx, const double* M, int m, int n, int kcap, SplitM
   if (e != cudaSuccess) return fail(ctx, XTRG_ECUDA, "svd split %dx%d: %s", m, n, cudaGetErrorString(e));
   if (!conv) return fail(ctx, XTRG_ENUMERIC, "Jacobi SVD of a %dx%d matrix did not converge", m, n);
   if (!std::isfinite(r->sigma_max)) return fail(ctx, XTRG_ENUMERIC, "non-finite singular value");
-  int len = m > n ? m : n, nc = m > n ? n : m;
-  ctx->flops_split += (double)r->sweeps * nc * (nc - 1) / 2.0 * (6.0 * len + 4.0 * nc);
+  // pivoted QR of q x p (a dot, an update and a norm for every column left after
+  // each of its c pivots), sweeps over pairs of its c columns of length p (a dot
+  // and three shears), the projection, the Gram of the isometry and its lower part
+  // times the projection
+  const double p = mode == SPLIT_RIGHT ? m : n, q = mode == SPLIT_RIGHT ? n : m, c = r->columns;
+  const double k = r->k;
+  ctx->flops_split += 6.0 * q * (c * p - c * (c + 1) / 2.0) + r->sweeps * c * (c - 1) / 2.0 * 8.0 * p +
+                      2.0 * p * q * k + 2.0 * p * k * k + q * k * (k - 1);
   return XTRG_OK;
 }
 
