@@ -16,13 +16,12 @@
 // FP32 Cholesky, all-SM triangular solve; see below), the second pass to first
 // order where that suffices.  A pivot that shows a column to be numerically
 // dependent on those before it drops the column: its output is zero (dead)
-// and the noise gives it a fresh direction in the next sweep.  (Block
-// Gram-Schmidt for such bases took 1.7 ms each at k = 256, for 45 of the 504
-// updates of a doubling at L = 64, D* = 256, and what it kept of a column that
-// failed the second pass was rounding noise: the errors of the free energy, the
-// energy and the magnetisation moment are the same without it, the doubling
-// 868 -> 800 ms.)  The caller checks max |U^T U - I| over the live columns and
-// takes the exact split when the FP32 products lost orthogonality.
+// and the noise gives it a fresh direction in the next sweep (CQ_TAU1,
+// CQ_TAU2).  Completing the bases that fail the second pass by block
+// Gram-Schmidt instead took 1.7 ms each at k = 256, for 45 of the 504 updates of
+// a doubling at L = 64, D* = 256 (868 ms, 790 without).  The caller checks
+// max |U^T U - I| over the live columns and takes the exact split when the FP32
+// products lost orthogonality.
 #include <math.h>
 #include <string.h>
 
@@ -206,6 +205,18 @@ cudaError_t tc_product(const View& a, const View& b, int M, int N, int K, float*
 // the columns before it (a warm start far from converged, a growing bond) and
 // is dropped; a column whose norm is zero is dead: their output columns are
 // zero.
+//
+// Thresholds of the scaled pivot, the squared part of a unit column that is
+// orthogonal to those before it.  First pass: the Gram's own error, up to 1e-6
+// at k = 256.  Second pass: its columns are nearly orthonormal, and one with a
+// small pivot is the remainder of a column that only just passed the first.
+// That remainder still carries weight; dividing it by its norm raises the 3e-6
+// of FP32 to 3e-6 / sqrt(pivot), which has to stay below the 1e-4 the caller
+// accepts: 0.01 leaves a factor of three.  At 0.25 the second pass dropped 3 %
+// more columns than the first had, and one sweep over random states (L = 8, D* =
+// 50 to 128, 400 of them) discarded 15 % more weight than with Gram-Schmidt (+- 5 %);
+// at 0.01 0.998 +- 0.045 of it, and at 1e-30 no less, but exact splits set in.
+constexpr float CQ_TAU1 = 1e-6f, CQ_TAU2 = 0.01f;
 constexpr int CQ_NT = 384;        // threads of the factor kernel (12 warps: up to 170 registers)
 constexpr int CQ_SOLVE_NT = 256;  // threads of the solve kernel (8 warps, one row each)
 
@@ -595,7 +606,7 @@ cudaError_t cholqr2_block(float* Yb, long long ldy, int rows, int w, float* tmp,
     RET(tc_product(f32_view(src, idx_plain(1), idx_plain(lds)),
                    f32_view(src, idx_plain(1), idx_plain(lds)), w, w, rows, b.out, w, b, st));
     note_launch();
-    cholqr_factor<<<1, CQ_NT, fsm, st>>>(b.out, w, pass == 0 ? 1e-6f : 0.25f,
+    cholqr_factor<<<1, CQ_NT, fsm, st>>>(b.out, w, pass == 0 ? CQ_TAU1 : CQ_TAU2,
                                          b.chol_L, b.chol_d, b.chol_li, b.chol_flag, nullptr);
     RET(cudaGetLastError());
     note_launch();
@@ -1052,7 +1063,7 @@ cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm,
   note_launch();
   sum_partials_kernel<<<grid_for((long long)k * k), 256, 0, st>>>(b.part, sp, k, k, G, k);
   note_launch();
-  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 1e-6f, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, CQ_TAU1, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
                                        nullptr);
   RET(cudaGetLastError());
   note_launch();
@@ -1069,7 +1080,7 @@ cudaError_t narrow_split(int m, int n, int k, int dir_right, const double* warm,
   RET(cudaGetLastError());
   // the full second pass, only if E was too large: U1 -> b.Q
   note_launch();
-  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, 0.25f, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
+  cholqr_factor<<<1, CQ_NT, fsm, st>>>(G, k, CQ_TAU2, b.chol_L, b.chol_d, b.chol_li, b.chol_flag,
                                        need_full);
   RET(cudaGetLastError());
   note_launch();
