@@ -273,6 +273,14 @@ __device__ __forceinline__ void store_chunk(const TcOutput& o, long long om, boo
   const int lane = threadIdx.x & 31;
   if (o.mode != TC_OUT_BF16P) {
     if (!valid) return;
+    float* d = o.f32 + om + col[0];
+    if (f.layout == 2 && ncols == 32 && ((uintptr_t)d & 15) == 0) {
+#pragma unroll
+      for (int q4 = 0; q4 < 8; ++q4)
+        reinterpret_cast<float4*>(d)[q4] =
+            make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+      return;
+    }
 #pragma unroll
     for (int jj = 0; jj < 32; ++jj)
       if (jj < ncols) store_out(o, om + col[jj], v[jj]);
