@@ -25,7 +25,8 @@
  * - Device memory: the library allocates nothing on the device.  The caller
  *   provides one device workspace of at least xtrg_workspace_bytes() bytes
  *   (256-byte aligned); it is borrowed until xtrg_destroy and never freed by
- *   the library.  The library allocates small host bookkeeping only.
+ *   the library.  The library allocates small host bookkeeping only (one
+ *   page of it page-locked, see xtrg_tc_gemm).
  * - Streams: every device operation is issued on the CUDA stream given to
  *   xtrg_create (a cudaStream_t passed as void*; NULL = legacy default
  *   stream).  Calls that return scalars or bond dimensions to the host
@@ -265,7 +266,14 @@ xtrg_status xtrg_set_graphs(xtrg_ctx* ctx, int on);
  * x1*y0; 6: + x0*y2 + x1*y1 + x2*y0); splitk > 1 splits K across CTAs and
  * sums the partials in FP64.  workspace: device memory of at least
  * xtrg_tc_gemm_workspace_bytes() bytes, 256-byte aligned.  Synchronises the
- * stream.  Returns XTRG_ETIMEOUT if a bounded device wait expired. */
+ * stream.  Returns XTRG_ETIMEOUT if a bounded device wait expired.  The first
+ * call of the process (of this function, xtrg_tc_gemm_nn or
+ * xtrg_tc_gemm_static) takes one page of page-locked host memory, kept until
+ * the process exits, for the error flags that calls read back; later calls
+ * and threads allocate nothing.  Like every call that synchronises, none of
+ * the three may run while a stream of any thread is captured in global mode.
+ * A device that the library has used cannot be reset (cudaDeviceReset) and
+ * used again. */
 size_t xtrg_tc_gemm_workspace_bytes(int M, int N, int K, int batch, int planes, int splitk);
 xtrg_status xtrg_tc_gemm(const double* A, const double* B, double* C, int M, int N, int K,
                          int batch, int planes, int nprod, int splitk, void* workspace,
@@ -292,6 +300,7 @@ xtrg_status xtrg_tc_gemm_nn(const double* A, const double* B, double* C, int M, 
  * larger sizes return XTRG_ENOMEM and do nothing.  The call allocates no
  * device memory.  The first call on a device looks up the array's device
  * address (with that device current), so make it before any stream capture.
+ * As for xtrg_tc_gemm, the process's first call takes a page-locked page.
  * Every call uses the same array: calls that overlap on the GPU race, so
  * order them (one stream, or events).  Uses the current device and
  * synchronises the given stream. */
