@@ -639,10 +639,11 @@ __global__ void subtract_block_kernel(float* __restrict__ Yb, long long ldy,
 // O(E^2), Phi(E) the strictly lower part of E plus half its diagonal, so
 // U2 = U1 L^{-T} = U1 (I - Phi(E)^T) + O(E^2) and U2^T U2 = I + O(E^2).
 // Writes B = I - Phi(E) (k x k: U2 = U1 B^T is one tensor-core product);
-// dead columns (G2_jj < 1/2, zero columns of U1) keep B's row e_j
-// and get zeros elsewhere.  If a live |E_ij| exceeds emax (or is not
-// finite), sets *need_full: the full second pass runs instead (and counts
-// itself in need_full[1]).
+// dead columns (zero columns of U1) keep B's row e_j and get zeros elsewhere.
+// If a live |E_ij| exceeds emax (or is not finite), or a column that is not zero
+// has lost half its norm (G2_jj < 1/2: the first order cannot restore it), sets
+// *need_full: the full second pass runs instead (and counts itself in
+// need_full[1]).
 // G comes as the partials of its split contraction: summed here, with the
 // sum written to G for the full second pass; B as its BF16 planes.
 __global__ void __launch_bounds__(256)
@@ -684,6 +685,7 @@ __global__ void __launch_bounds__(256)
     if (c < k) {
       if (!(gn >= 0.5f)) {
         v = (n == c) ? 1.f : 0.f;
+        if (n == c && gn != 0.f) big = true;
       } else if (gc >= 0.5f) {
         const float E = (n == c) ? gn - 1.f : g[u];
         if (!(fabsf(E) <= emax)) big = true;

@@ -67,12 +67,13 @@ def _doubled(b, dstar, prec, sweeps, fall=0.0, **kw):
     eng.close()
     C = _dense(out) * np.exp(lnc)
     # every site but the first is right-orthonormal on its live rows, to what a
-    # split may leave
+    # split may leave, and zero on the others
     for w in out[1:]:
         m = w.reshape(w.shape[0], -1)
         G = m @ m.T
         live = np.diag(G) > 0.5
         assert np.abs(G[np.ix_(live, live)] - np.eye(live.sum())).max() <= 1e-4
+        assert not m[~live].any()
     assert c["exact_split_fallbacks"] <= 0.1 * c["two_site_updates"]
     return P, C, o, out
 
@@ -97,7 +98,7 @@ def test_no_column_of_weight_is_lost(b, dstar, block, keep_parts):
     assert o["max_bond"] == dstar
 
 
-@pytest.mark.parametrize("b,dstar", [(8, 64), (9, 81), (11, 127), (13, 173)])
+@pytest.mark.parametrize("b,dstar", [(8, 64), (8, 65), (9, 81), (11, 127), (13, 173)])
 def test_three_products_lose_no_column_of_weight(b, dstar):
     """As above with operands of two planes, right to 2^-16: 4 L 2^-16 = 5e-4."""
     P, C, o, out = _doubled(b, dstar, "bf16x3", 2)
