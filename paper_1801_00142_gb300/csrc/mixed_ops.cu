@@ -110,6 +110,14 @@ PlaneJob<S> plane_job(const S* src, Idx3 rv, Idx3 kv, long long sbs, int rows, i
                       __nv_bfloat16* out, long long ld, long long obs, long long ops) {
   PlaneJob<S> j{};
   if ((long long)rows * ld * batch <= 0) return j;
+  // rows that follow one another across the batch are rows of one matrix: a tile
+  // holds 32 of them, whatever the size of the batch's matrices (500 of 1 x 4096:
+  // 111 -> 14 us; 2000 of 1 x 1 10.4 -> 5.1 us)
+  if (batch > 1 && rv.n1 == 1 && rv.n0 == 1 && sbs == rows * rv.s2 && obs == rows * ld &&
+      (long long)rows * batch <= 0x7fffffffLL) {
+    rows *= batch;
+    batch = 1;
+  }
   j.src = src; j.rv = rv; j.kv = kv; j.sbs = sbs; j.rows = rows; j.K = K;
   j.tiles_r = (rows + TP_R - 1) / TP_R;
   j.tiles_k = (int)((ld + TP_K - 1) / TP_K);

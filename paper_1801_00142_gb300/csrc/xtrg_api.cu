@@ -2019,13 +2019,21 @@ xtrg_status tc_gemm_run(const double* A, const double* B, double* C, int M, int 
   const TcOperand ob{pb, planes, N, K, lb.ld, lb.batch_stride, lb.plane_stride, batch, b_kn ? 1 : 0};
   TcOutput out;
   memset(&out, 0, sizeof out);
-  out.mode = splitk == 1 ? TC_OUT_F64 : TC_OUT_PARTIAL;
+  // An unsplit product is stored in FP64 by the epilogue.  With few rows only one
+  // warp of a tile's quarter has any, and at ragged N it stores value by value:
+  // where several such tiles an SM wait for it, FP32 partials and a pass that widens them
+  // are faster (5 x 300 x 7 of 500: 85 us, 74 so; 8 x 8 x 8 of 20000 357, 327; below
+  // four tiles an SM, or at 40 rows, the other way round).
+  const long long tiles = (long long)((M + 127) / 128) * ((N + 127) / 128) * batch;
+  const bool widen = splitk == 1 && M <= 32 && N % 32 != 0 && tiles >= 4 * 152;
+  out.mode = splitk == 1 && !widen ? TC_OUT_F64 : TC_OUT_PARTIAL;
   out.f32 = part;
   out.f64 = C;
   out.alpha = 1.0;
   if (tc_gemm(oa, ob, M, N, K, batch, nprod, splitk, out, err, st) != cudaSuccess)
     return XTRG_ECUDA;
-  if (splitk > 1 && reduce_partials(part, splitk, (long long)batch * M * N, C, st) != cudaSuccess)
+  if (out.mode == TC_OUT_PARTIAL &&
+      reduce_partials(part, splitk, (long long)batch * M * N, C, st) != cudaSuccess)
     return XTRG_ECUDA;
   PinnedFlag flag;
   int* h = flag.get();
