@@ -684,9 +684,11 @@ __global__ void __launch_bounds__(Epi<NPROD>::THREADS, 1)
                   make_double2(f32_to_f64(v[2 * q2]), f32_to_f64(v[2 * q2 + 1]));
           } else {
 #pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-              if (jj >= ncols) break;   // one branch past the last column, not one each
-              d[jj] = f32_to_f64(v[jj]);
+            for (int j0 = 0; j0 < 32; j0 += 4) {
+              if (j0 >= ncols) break;   // (a way out at every column spills two registers)
+#pragma unroll
+              for (int jj = j0; jj < j0 + 4; ++jj)
+                if (jj < ncols) d[jj] = f32_to_f64(v[jj]);
             }
           }
         } else if (o.mode == TC_OUT_PARTIAL) {
@@ -698,10 +700,8 @@ __global__ void __launch_bounds__(Epi<NPROD>::THREADS, 1)
                   make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
           } else {
 #pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-              if (jj >= ncols) break;   // one branch past the last column, not one each
-              d[jj] = v[jj];
-            }
+            for (int jj = 0; jj < 32; ++jj)
+              if (jj < ncols) d[jj] = v[jj];
           }
         } else {
 #pragma unroll
