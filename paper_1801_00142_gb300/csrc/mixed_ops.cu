@@ -91,8 +91,10 @@ __global__ void __launch_bounds__(256)
     const int y = tid / 8, z = tid % 8 * 8, r = r0 + y, k = k0 + z;
     if (r < j.rows && k < j.ld) {
       __nv_bfloat16* d = j.out + b * j.obs + (long long)r * j.ld + k;
-      for (int q = 0; q < planes; ++q, d += j.ops)
-        *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(&tp[q][y][z]);
+      // unrolled: without, 2^26 elements take 160 us
+#pragma unroll
+      for (int q = 0; q < 3; ++q, d += j.ops)
+        if (q < planes) *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(&tp[q][y][z]);
     }
     __syncthreads();
   }
