@@ -413,8 +413,6 @@ def run_native(args):
            "exact_split_fallbacks": s1["exact_split_fallbacks"] - s0["exact_split_fallbacks"],
            "truncation_ms_per_step": (p1["split_ms"] - p0["split_ms"]) / n_cycle,
            "tc_gemm_ms_per_step": tc_ms / n_cycle,
-           "orth_cluster_calls": s1["orth_cluster_calls"] - s0["orth_cluster_calls"],
-           "orth_fallbacks": s1["orth_fallbacks"] - s0["orth_fallbacks"],
            "orth_full_second_pass": s1["orth_full_second_pass"] - s0["orth_full_second_pass"],
            "orth_deflated_columns": s1["orth_deflated_columns"] - s0["orth_deflated_columns"],
            "graph_replays_timed": s1["graph_replays"] - s0["graph_replays"],

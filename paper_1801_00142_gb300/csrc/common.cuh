@@ -104,7 +104,8 @@ enum SplitMode { SPLIT_RIGHT = 0, SPLIT_LEFT = 1 };
 
 struct SvdResult {
   int k;              // kept singular values
-  int rank;           // singular values above rel_tol * sigma_max (before the cap)
+  int rank;           // singular values above rel_tol * sigma_max, before the cap (where kcap
+                      // cuts, of those in the QR's columns: above kcap if there are more)
   int columns;        // columns of the pivoted QR, which the sweeps run over
   int sweeps;         // Jacobi sweeps used
   double discarded;   // discarded weight / total weight

@@ -25,7 +25,7 @@ inline int grid_for(long long n) {
 // src (kfast: k, else the rows), the planes pass through shared memory, and
 // each thread writes eight consecutive columns of a row per plane, 16 bytes.
 // Every row starts 16-byte aligned: the launch refuses other layouts.
-// Measured on 2^26 FP64 elements, 3 planes (0.94 GB moved): 157 us, 88 % of
+// Measured on 2^26 FP64 elements, 3 planes (0.94 GB moved): 152 us, 91 % of
 // the measured copy rate; 862 us with an element a thread, its 64-bit divisions
 // and FP64 conversions.
 constexpr int TP_R = 32, TP_K = 64;
@@ -144,7 +144,7 @@ cudaError_t launch_to_planes(const PlaneJob<S>& j0, const PlaneJob<S>& j1, int p
   if (!rows_aligned(j0) || !rows_aligned(j1)) return cudaErrorInvalidValue;
   // two matrices share a launch while they leave room on the chip; larger ones
   // gain nothing by it, and the kernel of one has its view in constants (1024 x
-  // 65536: 157 us a matrix, 180 us in a pair)
+  // 65536: 152 us a matrix, 180 us in a pair)
   if (j0.tiles > 0 && j1.tiles > 0 && tiles > 152 * 16) {
     const cudaError_t e = launch_to_planes(j0, PlaneJob<S>{}, planes, clear, st, run_if, thresh);
     return e != cudaSuccess ? e : launch_to_planes(j1, PlaneJob<S>{}, planes, nullptr, st, run_if, thresh);

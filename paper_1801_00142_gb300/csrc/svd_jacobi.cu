@@ -41,8 +41,8 @@
 //     tau0 = 2^-26, against exact: 4e-8 without, 7e-16 with (the Hamiltonian is
 //     1e-8 of that state); it costs 1 % of a doubling at L = 32, D* = 40.
 //
-// GPU mapping: one kernel per split, one warp per column (step 1) or per
-// column pair of a round-robin round (step 2); columns live in L2 (read past
+// GPU mapping: one kernel per split, half a warp per column (step 1) or a warp
+// per column pair of a round-robin round (step 2); columns live in L2 (read past
 // L1).  Steps and rounds are separated by a barrier over all CTAs.  What
 // bounds it is latency: a step moves a few columns, does a hundred FP64
 // operations per lane pair and meets the barrier.  Small problems run in one
@@ -51,7 +51,7 @@
 // of FP64 (two FMAs a clock each), run as a cooperative grid with a bounded
 // barrier (on expiry the kernel records a timeout and every CTA leaves).
 // Measured, one FP64 doubling at L = 32, D* = 40, one sweep (62 splits of up
-// to 160 x 160): 965 ms with Jacobi on C_E, 108 ms with this split (an average
+// to 160 x 160): 1095 ms with Jacobi on C_E, 116 ms with this split (an average
 // split of its bulk takes 0.66 ms: 90 QR steps and some 400 rounds).
 #include <math.h>
 

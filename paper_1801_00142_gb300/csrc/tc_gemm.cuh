@@ -46,7 +46,8 @@ struct TcOutput {
   double alpha;
 };
 
-// C[b] = alpha * sum_products A[b] * B[b]^T (A: M x K, B: N x K, both K-major).
+// C[b] = alpha * sum_products A[b] * B[b]^T (A: M x K, B: N x K, both K-major);
+// TC_OUT_PARTIAL and TC_OUT_F64 leave alpha out (their callers have 1).
 // nprod in {1, 3, 6}; splitk >= 1 (only with TC_OUT_PARTIAL).
 cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int N, int K, int batch,
                     int nprod, int splitk, const TcOutput& out, int* dev_err, cudaStream_t st);
