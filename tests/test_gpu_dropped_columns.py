@@ -20,9 +20,9 @@ def _random_state(L, D, seed, fall):
 def test_second_pass_drops_no_more_than_rounding():
     """A column dropped in the second orthonormalisation pass is a bond
     direction lost, for good in the last sweep.  The count to meet, 7442 over
-    these 100 doublings of one sweep, is of the build in which Gram-Schmidt
+    these 100 doublings of one sweep, was taken when Gram-Schmidt still
     completed every basis that failed the second pass, so that only the first
-    pass dropped columns.  Two builds of that rule differ by the rounding of
+    pass dropped columns.  Two codes with that rule differ by the rounding of
     pivots at the threshold: by 2.6 columns a doubling (standard deviation, 400
     of them), 26 over 100; three times that is the allowance."""
     torch = pytest.importorskip("torch")
